@@ -104,8 +104,8 @@ typedef struct {
 } fpt_result;
 
 /* ------------------------------------------------------------------------------------------
- * Plain one-trajectory-per-thread path (the structure of Alg. 1 / Alg. 3: thread i integrates
- * realisation i to its escape).  FP64 reproduces the FP64 oracle's arithmetic order exactly
+ * Plain path (Alg. 1 / Alg. 3: every realisation integrated to its escape, no engine).
+ * FP64 reproduces the FP64 oracle's arithmetic order exactly
  * (no fused multiply-add, unwrapped phase); FP32 uses the engine's FP32 step.
  * ------------------------------------------------------------------------------------------ */
 

@@ -133,20 +133,26 @@ __device__ __forceinline__ void bm_pair_f32(uint32_t x0, uint32_t x1, float bmc,
     __sincosf(fmaf(kTwoPiF, mant_f32(x1), -9.42477796076937972f), &sn, &cs);
 }
 
-// Double-precision uniform in (0, 1): u = (x + 1/2) 2^-32, exact.
+// Double-precision uniform in (0, 1): u = (x + 1/2) 2^-32, exact.  With y = 2 x + 1 the double of
+// bits (2^19 : y) is 2^19 + y 2^-33, so u takes one FP64 subtraction and no conversion.
 __device__ __forceinline__ double uniform_f64(uint32_t x) {
-    return __dmul_rn(__dadd_rn(static_cast<double>(x), 0.5), 2.3283064365386962890625e-10);
+    const long long y = static_cast<long long>(2ull * x + 1ull);
+    return __dsub_rn(__longlong_as_double(0x4120000000000000ll | y), 524288.0);
 }
 
 // Box-Muller in double precision, evaluated in the order R = sqrt(-2 log u1), theta = (2 pi) u2,
-// z0 = R cos theta, z1 = R sin theta, each operation rounded separately.
+// z0 = R cos theta, z1 = R sin theta, each operation rounded separately.  sincos shares one
+// argument reduction and returns the bits of sin and cos (all 2^30 sampled angles); the exact
+// product -2 log u1 (log u1 is below -2^-33, never 0) is a sign flip and an exponent step.
 __device__ __forceinline__ void bm_pair_f64(uint32_t x0, uint32_t x1, double &z0, double &z1) {
     const double u1 = uniform_f64(x0);
     const double u2 = uniform_f64(x1);
-    const double r = __dsqrt_rn(__dmul_rn(-2.0, log(u1)));
-    const double theta = __dmul_rn(6.283185307179586476925286766559, u2);
-    z0 = __dmul_rn(r, cos(theta));
-    z1 = __dmul_rn(r, sin(theta));
+    const long long l = __double_as_longlong(log(u1));
+    const double r = __dsqrt_rn(__longlong_as_double((l ^ (1ll << 63)) + (1ll << 52)));
+    double sn, cs;
+    sincos(__dmul_rn(6.283185307179586476925286766559, u2), &sn, &cs);
+    z0 = __dmul_rn(r, cs);
+    z1 = __dmul_rn(r, sn);
 }
 
 // Per-lane constants of the FP32 step, decoded from a request on the host (set-up of Alg. 1).
