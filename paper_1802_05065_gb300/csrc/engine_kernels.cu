@@ -84,10 +84,6 @@ __device__ __forceinline__ void set_idle(Lane &L) {
     L.dt = L.A = L.amp = L.bmc = L.nudt = L.gb = L.Jf = 0.0f;
 }
 
-__device__ __forceinline__ unsigned clamp_u32(unsigned long long x) {
-    return x > 0xFFFFFFFFull ? 0xFFFFFFFFu : static_cast<unsigned>(x);
-}
-
 // Request constants and the trajectory's Philox stream; gid and the block count c are set.
 __device__ __forceinline__ void load_consts(Lane &L, const SlotDev *S) {
     L.dt = S->dt;
@@ -139,8 +135,9 @@ __device__ __forceinline__ void init_lane(Lane &L, const EngineDev &E, int s, un
     L.budget = S->budget0;
 }
 
-// Continue a suspended trajectory exactly where it stopped.
-__device__ __forceinline__ void resume_lane(Lane &L, const EngineDev &E, int s, const ParkEntry &P) {
+// Continue a trajectory exactly where it stopped (a suspended one, or one that changes warps).
+template <typename State>
+__device__ __forceinline__ void resume_from(Lane &L, const EngineDev &E, int s, const State &P) {
     const SlotDev *S = E.slots + s;
     L.slot = s;
     L.r = P.r;
@@ -184,6 +181,10 @@ struct CtaView {
     unsigned long long *res_base;   // ... and first id (ids res_base .. res_base + res_cnt - 1)
     int *started;                // per warp: trajectories it started in this launch
     int *pool;                   // blocks of this launch not yet taken by a warp of the CTA
+    int *warp_act, *warp_knd;    // per warp: lanes with a trajectory, and their kind
+    unsigned *share;             // blocks of the launch every warp runs before it takes from the pool
+    int *tail;                   // 1: the CTA's warps meet to run its last trajectories together
+    int tail_groups;             // groups of 32 lanes the CTA can run that way (0: it never does)
 };
 
 // Publish the trajectories finishing in this warp at this block end (warp-collective: every lane
@@ -193,7 +194,7 @@ struct CtaView {
 // it does not wait for, and gives back the group's in-flight places.  Histogram counts are
 // grouped by (slot, id block, bin) the same way.  The scan kernel reads the id blocks only
 // after the launch, so the order of the additions is free.
-__device__ __forceinline__ void emit_warp(const EngineDev &E, const CtaView &V, bool fin, int slot,
+__device__ __forceinline__ void emit_warp(const EngineDev &E, int *held, bool fin, int slot,
                                           unsigned long long gid, bool escaped, unsigned long long k) {
     const int lane = threadIdx.x & 31;
     // an index out of range (checked build only) drops the trajectory's result
@@ -263,7 +264,7 @@ __device__ __forceinline__ void emit_warp(const EngineDev &E, const CtaView &V, 
     const int n = __popc(grp);
     atomicAdd(&A->done, static_cast<unsigned>(n));
     atomicSub(&E.ctl[slot].inflight, n);
-    atomicSub(&V.held[slot], n);
+    atomicSub(&held[slot], n);
 }
 
 // Rare per-lane path: the phase reached hb = min(eb, pi), where eb = phi* - 2 pi w is the
@@ -292,9 +293,30 @@ __device__ __forceinline__ void wrap_down(Lane &L, const EngineDev &E) {
     L.hb = fminf(fmaf(-kTwoPiF, static_cast<float>(L.w - S->w0), S->eb0), kPiF);
 }
 
+// At the end of a block in which lane L escaped or its countdown ran out: true when the trajectory
+// is finished, with its step in `k` if it escaped within its budget; otherwise the bias is
+// re-based.  `useful` (the caller counted whole blocks) loses the steps past the end.
+__device__ __forceinline__ bool finished(Lane &L, const EngineDev &E, bool &escaped, unsigned long long &k,
+                                         unsigned long long &useful) {
+    const SlotDev *S = E.slots + L.slot;
+    const unsigned long long c = lane_c(L);
+    const unsigned long long max_steps = S->max_steps;
+    if (L.esc < 0 && c < S->nblocks) {   // re-base of the bias, not the end of the budget
+        set_progress(L, S);
+        return false;
+    }
+    if (L.esc >= 0) {
+        k = 4ull * (c - kBlockPhilox) + static_cast<unsigned long long>(L.esc) + 1ull;
+        escaped = k <= max_steps;
+    }
+    if (escaped) useful -= static_cast<unsigned long long>(kBlockSteps - 1 - L.esc);
+    else useful -= 4ull * c - max_steps;
+    return true;
+}
+
 // Finish lanes that escaped in the last block or reached the step budget (warp-collective).
 template <int T>
-__device__ __forceinline__ void finish_lanes(Lane (&L)[T], const EngineDev &E, const CtaView &V,
+__device__ __forceinline__ void finish_lanes(Lane (&L)[T], const EngineDev &E, int *held,
                                              unsigned long long &useful, int &n_active, unsigned &n_esc,
                                              unsigned &n_cens) {
 #pragma unroll
@@ -304,23 +326,10 @@ __device__ __forceinline__ void finish_lanes(Lane (&L)[T], const EngineDev &E, c
         if (L[t].slot < 0) {
             L[t].budget = 0xFFFFFFFFu;
         } else if (L[t].esc >= 0 || L[t].budget == 0) {
-            const SlotDev *S = E.slots + L[t].slot;
-            const unsigned long long c = lane_c(L[t]);
-            const unsigned long long max_steps = S->max_steps;
-            if (L[t].esc < 0 && c < S->nblocks) {   // re-base of the bias, not the end of the budget
-                set_progress(L[t], S);
-            } else {
-                fin = true;
-                if (L[t].esc >= 0) {
-                    k = 4ull * (c - kBlockPhilox) + static_cast<unsigned long long>(L[t].esc) + 1ull;
-                    escaped = k <= max_steps;
-                }
-                if (escaped) useful -= static_cast<unsigned long long>(kBlockSteps - 1 - L[t].esc);
-                else useful -= 4ull * c - max_steps;
-            }
+            fin = finished(L[t], E, escaped, k, useful);
         }
         const unsigned long long gid = (static_cast<unsigned long long>(L[t].gid_hi) << 32) | L[t].gid_lo;
-        emit_warp(E, V, fin, L[t].slot, gid, escaped, k);
+        emit_warp(E, held, fin, L[t].slot, gid, escaped, k);
         if (fin) {
             if (escaped) ++n_esc;
             else ++n_cens;
@@ -338,10 +347,11 @@ __device__ __forceinline__ void finish_lanes(Lane (&L)[T], const EngineDev &E, c
 // nobody waits for).  While some request is
 // starved (strict caps, set by the host with preemption orders) each request is kept within
 // this CTA's share of its fair-share cap, counted in shared memory; otherwise lanes take work
-// from the first request that has some, so no lane idles while any request has work.
+// from the first request that has some, so no lane idles while any request has work.  Returns the
+// lanes that stay idle.
 template <int T>
-__device__ __forceinline__ void refill(Lane (&L)[T], const EngineDev &E, const CtaView &V, int kind,
-                                       int &n_active, unsigned &cursor, unsigned b) {
+__device__ __forceinline__ int refill(Lane (&L)[T], const EngineDev &E, const CtaView &V, int kind,
+                                      int &n_active, unsigned &cursor, unsigned b) {
     const int lane = threadIdx.x & 31;
     const unsigned lt = (1u << lane) - 1u;
     unsigned idle[T];
@@ -351,11 +361,11 @@ __device__ __forceinline__ void refill(Lane (&L)[T], const EngineDev &E, const C
         idle[t] = __ballot_sync(kFull, L[t].slot < 0);
         total += __popc(idle[t]);
     }
-    if (total == 0) return;
-    if (static_cast<int>(threadIdx.x >> 5) >= *E.claim_warps) return;   // spread scarce work
-    if (!checked(E, kind >= 0 && kind < kNumKinds, kChkKind)) return;
+    if (total == 0) return 0;
+    if (static_cast<int>(threadIdx.x >> 5) >= *E.claim_warps) return total;   // spread scarce work
+    if (!checked(E, kind >= 0 && kind < kNumKinds, kChkKind)) return total;
     const int cnt = E.act_count[kind];
-    if (cnt <= 0) return;
+    if (cnt <= 0) return total;
     const int *list = E.act_list + kind * E.max_requests;
     const bool capped = *E.strict != 0;
     const int wl = static_cast<int>(threadIdx.x >> 5);
@@ -462,7 +472,7 @@ __device__ __forceinline__ void refill(Lane (&L)[T], const EngineDev &E, const C
                 if (((m >> lane) & 1u) && rank < got) {
                     if (rank < gp) {
                         const unsigned pi = (p0 + static_cast<unsigned>(rank)) % S->park_cap;
-                        if (checked(E, pi < S->park_cap, kChkPark)) resume_lane(L[t], E, s, S->park[pi]);
+                        if (checked(E, pi < S->park_cap, kChkPark)) resume_from(L[t], E, s, S->park[pi]);
                     } else if (rank < gp + rt) {
                         init_lane(L[t], E, s, rb + static_cast<unsigned long long>(rank - gp));
                     } else {
@@ -474,8 +484,10 @@ __device__ __forceinline__ void refill(Lane (&L)[T], const EngineDev &E, const C
                 idle[t] = __ballot_sync(kFull, L[t].slot < 0);
             }
             total -= got;
+            if (total == 0 && lane == 0) V.warp_act[wl] = 32;
         }
     }
+    return total;
 }
 
 // Integrate blocks of kBlockSteps steps with model M, integrator H and bias kind R (constant or
@@ -500,6 +512,50 @@ __device__ __forceinline__ bool grant(const CtaView &V, unsigned &limit) {
     return g > 0;
 }
 
+// This warp's lanes after an event, for the CTA's view, and whether the CTA has run dry
+// (warp-collective): nothing left to claim or resume in any listed request, no reservoir, and few
+// enough trajectories left for its groups.  Then the warps are called together (V.tail); the
+// exact counts are taken when they have met.
+template <int T>
+__device__ __forceinline__ void look_dry(Lane (&L)[T], const EngineDev &E, const CtaView &V, int kind) {
+    if constexpr (T == 1) {
+        if (V.tail_groups == 0) return;
+        const int lane = threadIdx.x & 31, warps = static_cast<int>(blockDim.x >> 5);
+        const int act = __popc(__ballot_sync(kFull, L[0].slot >= 0));
+        if (lane == 0) {
+            V.warp_act[threadIdx.x >> 5] = act;
+            V.warp_knd[threadIdx.x >> 5] = kind;
+        }
+        __syncwarp();
+        const int a = lane < warps ? vload(V.warp_act[lane]) : 0;
+        const int total = __reduce_add_sync(kFull, a);
+        const int kinds = __popc(__reduce_or_sync(kFull, a > 0 ? 1u << (vload(V.warp_knd[lane]) & 31) : 0u));
+        // groups: ceil(lanes / 32) of one kind, at most (lanes + 31 kinds) / 32 of several
+        if (total == 0 || total + (kinds > 1 ? 31 * kinds : 0) > 32 * V.tail_groups) return;
+        bool work = lane < warps && vload(V.res_cnt[lane]) > 0;
+        for (int k = 0; k < kNumKinds; ++k)
+            for (int j = lane; j < E.act_count[k]; j += 32)
+                work |= (vload(V.ok[E.act_list[k * E.max_requests + j]]) & 3u) != 0u;
+        if (!__any_sync(kFull, work) && lane == 0) *V.tail = 1;
+    }
+}
+
+// Blocks this warp may run before it looks again whether the CTA's warps are called together (a
+// look per block costs 2 % of a full CTA's rate).
+constexpr unsigned kLookBlocks = 32;
+
+// More blocks for this warp (warp-collective): its own share kLookBlocks at a time, then the
+// CTA's pool; false when there are none or the warps are called together.
+__device__ __forceinline__ bool more(const CtaView &V, unsigned &limit) {
+    if (vload(*V.tail) != 0) return false;
+    const unsigned share = *V.share;
+    if (limit < share) {
+        limit = limit + kLookBlocks < share ? limit + kLookBlocks : share;
+        return true;
+    }
+    return grant(V, limit);
+}
+
 template <int M, int H, int R, int T>
 __device__ __forceinline__ unsigned run_blocks(Lane (&L)[T], const EngineDev &E, const CtaView &V, unsigned b,
                                                int &n_active,
@@ -514,7 +570,7 @@ __device__ __forceinline__ unsigned run_blocks(Lane (&L)[T], const EngineDev &E,
 #pragma unroll
     for (int t = 0; t < T; ++t)
         if constexpr (!R) bias_line(fmaf(L[t].nudt, L[t].Jf, L[t].gb), L[t].nudt, L[t].dt, gs[t], gsl[t]);
-    while (b < limit || grant(V, limit)) {
+    while (b < limit || more(V, limit)) {
         // the block's normals: Philox blocks c .. c + kBlockPhilox - 1 (c is a multiple of
         // kBlockPhilox, so c_lo + h never carries into c_hi)
         float rr[T][2 * kBlockPhilox], tg[T][kBlockSteps];
@@ -586,8 +642,9 @@ __device__ __forceinline__ unsigned run_blocks(Lane (&L)[T], const EngineDev &E,
                     philox_lane_init(L[t].P, S->key0, S->key1, L[t].c_hi, L[t].gid_lo, L[t].gid_hi);
                 }
             }
-            finish_lanes(L, E, V, useful, n_active, n_esc, n_cens);
-            refill(L, E, V, kind_of(M, H, R), n_active, cursor, b);
+            finish_lanes(L, E, V.held, useful, n_active, n_esc, n_cens);
+            const int idle = refill(L, E, V, kind_of(M, H, R), n_active, cursor, b);
+            if (idle > 0) look_dry(L, E, V, kind_of(M, H, R));
             if (!__any_sync(kFull, n_active > 0)) break;
             if constexpr (!R) {
 #pragma unroll
@@ -618,8 +675,430 @@ __device__ __forceinline__ int seek_work(Lane (&L)[T], const EngineDev &E, const
     return -1;
 }
 
+// ---- the CTA's last trajectories -----------------------------------------------------------
+// When a CTA has nothing left to claim, its lanes thin out while its warps keep their issue
+// slots: a warp with one lane costs what a full one does, and a full CTA takes 82 ns per step.
+// One warp alone on a scheduler still takes 31 ns per step, of which the chain phase -> sin ->
+// phase is 14 ns and the rest the noise made in front of it.  So the CTA's warps meet, the
+// remaining trajectories are packed into the fewest groups of 32 lanes of one kind, and each group
+// gets one warp that only integrates and three that only make its noise: chunks of blocks of 16
+// steps through a ring of three chunks in shared memory, one named barrier of the group per chunk
+// (the noise is two chunks ahead, so the next block's loads never wait).  Integrating takes ~8
+// cycles of a scheduler per step and noise ~27, so the integrating warps sit on one scheduler (warp
+// index mod 4) and the noise on the other three: beside a noise warp the chain waits for the MUFU
+// and multiply pipes (measured in a loop of these parts alone, four groups with two noise warps:
+// 26 ns per step mixed).  After each round of kRoundBlocks blocks or more the groups
+// are packed again if that makes them fewer.  The arithmetic of a trajectory is that of
+// run_blocks, bit for bit.  ns per step at 1 / 2 / 3 / 4 full warps per SM, the plain loop -> this:
+// overdamped Euler 31.5 / 31.5 / 31.5 / 31.5 -> 18.5 / 20.2 / 22.1 / 24.8, underdamped ramped Euler
+// 30.4 / 30.5 / 30.5 / 30.5 -> 14.8 / 18.8 / 22.8 / 27.5, underdamped Heun 40 -> 25 / 26 / 31 / 33;
+// a request of 1024 trajectories of 19 000 steps 3.7 -> 2.3 ms.
+constexpr int kTailGroupsMax = 5;       // a quarter of the warps: one scheduler's
+constexpr int kTailMakers = 3;          // noise warps per group
+constexpr int kTailChunk = 3;           // blocks per chunk, one for each of them
+constexpr int kTailRing = 3 * kTailChunk;                     // blocks in a group's ring
+constexpr int kRoundBlocks = 256;
+constexpr int kNoiseFloats = 24;                              // per lane and block: 8 radii, 16 cos / sin
+constexpr int kNoiseBlock = 32 * kNoiseFloats;                // floats of one block of a group
+constexpr int kTailMinWarps = 8;
+
+struct TailLane {      // a trajectory while it changes warps, or its result
+    float r, v;
+    int w, slot;
+    unsigned c_lo, c_hi, gid_lo, gid_hi;   // result: c is the escape step
+    int fin;                               // kTailRuns, kTailEscaped or kTailCensored
+};
+enum : int { kTailRuns = 0, kTailEscaped = 1, kTailCensored = 2 };
+
+// Groups a CTA of `warps` warps takes on; CTAs below kTailMinWarps warps do without.
+__host__ __device__ constexpr int tail_groups_of(int T, int warps) {
+    return T != 1 || warps < kTailMinWarps ? 0 : (warps / 4 < kTailGroupsMax ? warps / 4 : kTailGroupsMax);
+}
+constexpr size_t tail_shared_bytes(int warps) {
+    return tail_groups_of(1, warps) == 0 ? 0 : static_cast<size_t>(tail_groups_of(1, warps)) * kTailRing * kNoiseBlock * 4 +
+                                               kTailGroupsMax * 32 * sizeof(TailLane);
+}
+
+__device__ __forceinline__ void group_barrier(int group) {
+    asm volatile("bar.sync %0, %1;" ::"r"(group + 1), "n"(32 * (1 + kTailMakers)) : "memory");
+}
+
+// One block of noise of one lane: tg[h] of call h at float4 (h, lane), its two radii at
+// float2 (h, lane) behind them.
+__device__ __forceinline__ void noise_store(float *block, int lane, int h, float2 rr, float4 tg) {
+    reinterpret_cast<float4 *>(block)[32 * h + lane] = tg;
+    reinterpret_cast<float2 *>(block + 16 * 32)[32 * h + lane] = rr;
+}
+__device__ __forceinline__ void noise_load(const float *block, int lane, int h, float2 &rr, float4 &tg) {
+    tg = reinterpret_cast<const float4 *>(block)[32 * h + lane];
+    rr = reinterpret_cast<const float2 *>(block + 16 * 32)[32 * h + lane];
+}
+
+// Steps of call h of a block (4 h .. 4 h + 3).
+template <int M, int H, int R, typename F>
+__device__ __forceinline__ void four_steps(Lane &L, int h, float2 rr, float4 tg, float gs, float gsl, F after) {
+    const float t[4] = {tg.x, tg.y, tg.z, tg.w};
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int s = 4 * h + q;
+        step_f32<M, H>(L.r, L.v, q < 2 ? rr.x : rr.y, t[q], bias_b0<H, R>(gs, gsl, s), bias_b1<H, R>(gs, gsl, s),
+                       L.dt, L.A, L.amp);
+        after(s);
+    }
+}
+
+static_assert(kTailGroupsMax <= kNumKinds, "the packing keeps the groups' kinds in count[]");
+// The packed lanes and, behind them, the noise of the groups (a CTA's dynamic shared memory).
+extern __shared__ __align__(16) unsigned char tail_mem[];
+__device__ __forceinline__ TailLane *tail_lanes() { return reinterpret_cast<TailLane *>(tail_mem); }
+__device__ __forceinline__ float *tail_group_noise(int group) {
+    return reinterpret_cast<float *>(tail_mem + kTailGroupsMax * 32 * sizeof(TailLane)) + group * kTailRing * kNoiseBlock;
+}
+struct TailShared {
+    int count[kNumKinds];                   // lanes per kind (of the packing that is under way)
+    int kind[kTailGroupsMax];               // of each group
+    int alive[kTailGroupsMax];              // its lanes with a trajectory, after a round
+    int stop[2][kTailGroupsMax];            // group done, by parity of the chunk
+};
+__shared__ TailShared tail_sh;
+
+// Groups of 32 lanes of one kind that the CTA's trajectories make (CTA-collective); `base` gets
+// the place of this warp's first lane among the lanes of its kind, `at` its kind's first group.
+__device__ __forceinline__ int tail_count(Lane (&L)[1], int (&count)[kNumKinds], int kind, int &base, int &at) {
+    __syncthreads();
+    if (threadIdx.x < kNumKinds) count[threadIdx.x] = 0;
+    __syncthreads();
+    const unsigned held = __ballot_sync(kFull, L[0].slot >= 0);
+    base = 0;
+    if (held) {
+        if ((threadIdx.x & 31) == 0) base = atomicAdd(&count[kind], __popc(held));
+        base = __shfl_sync(kFull, base, 0);
+    }
+    __syncthreads();
+    int groups = 0;
+    at = 0;
+    for (int k = 0; k < kNumKinds; ++k) {
+        if (k == kind) at = groups;
+        groups += (count[k] + 31) >> 5;
+    }
+    return groups;
+}
+
+// Lane state between launches.
+__device__ __forceinline__ void store_lane(const EngineDev &E, unsigned i, const Lane &L) {
+    if (!checked(E, i < E.n_lanes, kChkLane)) return;
+    E.lanes.slot[i] = L.slot;
+    if (L.slot < 0) return;
+    E.lanes.r[i] = L.r;
+    E.lanes.v[i] = L.v;
+    E.lanes.hb[i] = L.hb;
+    E.lanes.w[i] = L.w;
+    E.lanes.c_lo[i] = L.c_lo;
+    E.lanes.c_hi[i] = L.c_hi;
+    E.lanes.gid_lo[i] = L.gid_lo;
+    E.lanes.gid_hi[i] = L.gid_hi;
+}
+__device__ __forceinline__ void load_lane(Lane &L, const EngineDev &E, unsigned i, int s) {
+    const SlotDev *S = E.slots + s;
+    L.slot = s;
+    L.r = E.lanes.r[i];
+    L.v = E.lanes.v[i];
+    L.hb = E.lanes.hb[i];
+    L.w = E.lanes.w[i];
+    L.c_lo = E.lanes.c_lo[i];
+    L.c_hi = E.lanes.c_hi[i];
+    L.gid_lo = E.lanes.gid_lo[i];
+    L.gid_hi = E.lanes.gid_hi[i];
+    L.esc = -1;
+    load_consts(L, S);
+    set_progress(L, S);
+}
+
+// A warp's share of the launch's counters (warp-collective).
+__device__ __forceinline__ void add_counters(const EngineDev &E, unsigned long long useful, unsigned n_esc, unsigned n_cens) {
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        useful += __shfl_down_sync(kFull, useful, off);
+        n_esc += __shfl_down_sync(kFull, n_esc, off);
+        n_cens += __shfl_down_sync(kFull, n_cens, off);
+    }
+    if ((threadIdx.x & 31) == 0) {
+        if (useful) atomicAdd(&E.counters[kCntUseful], useful);
+        if (n_esc) atomicAdd(&E.counters[kCntEscapes], static_cast<unsigned long long>(n_esc));
+        if (n_cens) atomicAdd(&E.counters[kCntCensored], static_cast<unsigned long long>(n_cens));
+    }
+}
+
+// One round of a group's integrating warp: its lanes from shared memory and back, results left
+// there.  A call's registers are loaded with the next block's noise
+// as soon as its steps are done, so the loads are off the chain; the rare replay reads its block
+// again.
+template <int M, int H, int R>
+__device__ __forceinline__ void tail_integrate(const EngineDev &E, int group, int round) {
+    const int lane = threadIdx.x & 31;
+    const float *noise = tail_group_noise(group);
+    TailShared &sh = tail_sh;
+    unsigned long long useful = 0;
+    unsigned n_esc = 0, n_cens = 0;
+    Lane L;
+    TailLane &T = tail_lanes()[32 * group + lane];
+    set_idle(L);
+    L.c_lo = 0u;
+    if (T.slot >= 0) resume_from(L, E, T.slot, T);
+    int n_active = L.slot >= 0 ? 1 : 0;
+    float gs, gsl;
+    bias_line(fmaf(L.nudt, L.Jf, L.gb), L.nudt, L.dt, gs, gsl);
+    const float *end = noise + kTailRing * kNoiseBlock, *cur = noise;   // this block's noise
+    float2 rr[kBlockPhilox];
+    float4 tg[kBlockPhilox];
+    group_barrier(group);
+#pragma unroll
+    for (int h = 0; h < kBlockPhilox; ++h) noise_load(cur, lane, h, rr[h], tg[h]);
+    int b = 0, b_count = 0, left = kTailChunk;   // blocks done, blocks counted, blocks left of the chunk
+    for (int parity = 0;;) {
+        if constexpr (R) bias_line(fmaf(L.nudt, L.Jf, L.gb), L.nudt, L.dt, gs, gsl);
+        const float *next = cur + kNoiseBlock == end ? noise : cur + kNoiseBlock;
+        const float r0 = L.r, v0 = L.v;
+        float mx = -INFINITY;
+#pragma unroll
+        for (int h = 0; h < kBlockPhilox; ++h) {
+            four_steps<M, H, R>(L, h, rr[h], tg[h], gs, gsl, [&](int) { mx = fmaxf(mx, L.r); });
+            noise_load(next, lane, h, rr[h], tg[h]);
+        }
+        L.c_lo += kBlockPhilox;
+        if constexpr (R) L.Jf += static_cast<float>(kBlockSteps);
+        L.budget -= 1u;
+        ++b;
+        bool over = false;
+        if (__any_sync(kFull, mx >= L.hb || L.budget == 0u || L.r < -kPiF)) {
+            useful += static_cast<unsigned long long>(kBlockSteps) * static_cast<unsigned>(n_active * (b - b_count));
+            b_count = b;
+            if (mx >= L.hb) {
+                L.r = r0;
+                L.v = v0;
+#pragma unroll
+                for (int h = 0; h < kBlockPhilox; ++h) {
+                    float2 rr2;
+                    float4 tg2;
+                    noise_load(cur, lane, h, rr2, tg2);
+                    four_steps<M, H, R>(L, h, rr2, tg2, gs, gsl, [&](int s) {
+                        if (L.r >= L.hb) phase_event(L, E, s);
+                    });
+                }
+            }
+            if (L.r < -kPiF) wrap_down(L, E);
+            if (L.slot >= 0 && L.c_lo == 0u) L.c_hi += 1u;   // 2^32-block carry
+            if (L.slot >= 0 && (L.esc >= 0 || L.budget == 0u)) {
+                bool escaped = false;
+                unsigned long long k = 0ull;
+                if (finished(L, E, escaped, k, useful)) {
+                    T.fin = escaped ? kTailEscaped : kTailCensored;
+                    T.c_lo = static_cast<unsigned>(k);
+                    T.c_hi = static_cast<unsigned>(k >> 32);
+                    if (escaped) ++n_esc;
+                    else ++n_cens;
+                    set_idle(L);
+                    n_active = 0;
+                }
+            } else if (L.slot < 0) {
+                L.budget = 0xFFFFFFFFu;
+            }
+            over = !__any_sync(kFull, n_active > 0);
+            if constexpr (!R) bias_line(fmaf(L.nudt, L.Jf, L.gb), L.nudt, L.dt, gs, gsl);
+        }
+        cur = next;
+        if (--left == 0 || b == round || over) {
+            // Every warp of the group passes the same barriers: the verdict on a chunk lies in the
+            // slot of its parity, written again only after the barrier that follows.
+            if (lane == 0) sh.stop[parity][group] = over ? 1 : 0;
+            group_barrier(group);
+            if (over || b == round) break;
+            parity ^= 1;
+            left = kTailChunk;
+        }
+    }
+    useful += static_cast<unsigned long long>(kBlockSteps) * static_cast<unsigned>(n_active * (b - b_count));
+    if (L.slot >= 0) {
+        T.r = L.r;
+        T.v = L.v;
+        T.w = L.w;
+        T.c_lo = L.c_lo;
+        T.c_hi = L.c_hi;
+    }
+    const int alive = __popc(__ballot_sync(kFull, L.slot >= 0));
+    if (lane == 0) sh.alive[group] = alive;
+    add_counters(E, useful, n_esc, n_cens);
+}
+
+// One round of one of a group's noise warps: block `rank` of every chunk, two chunks ahead of the
+// integrating warp.
+__device__ __forceinline__ void tail_noise(const EngineDev &E, int group, int rank, int round) {
+    const int lane = threadIdx.x & 31;
+    float *ring = tail_group_noise(group);
+    const TailLane &T = tail_lanes()[32 * group + lane];
+    unsigned key0 = 0u, key1 = 0u, gid_lo = 0u, gid_hi = 0u, lo = 0u, hi = 0u;
+    float bmc = 0.0f;
+    if (T.slot >= 0) {
+        const SlotDev *S = E.slots + T.slot;
+        key0 = S->key0;
+        key1 = S->key1;
+        bmc = S->bmc;
+        gid_lo = T.gid_lo;
+        gid_hi = T.gid_hi;
+        const unsigned long long c = ((static_cast<unsigned long long>(T.c_hi) << 32) | T.c_lo) +
+                                     static_cast<unsigned>(kBlockPhilox * rank);
+        lo = static_cast<unsigned>(c);
+        hi = static_cast<unsigned>(c >> 32);
+    }
+    PhiloxLane P;
+    philox_lane_init(P, key0, key1, hi, gid_lo, gid_hi);
+    // keep the round keys in registers: formed again at each use they cost four instructions per step
+#pragma unroll
+    for (int r = 0; r < 8; ++r) asm volatile("" : "+r"(P.ka[r]));
+#pragma unroll
+    for (int r = 0; r < 7; ++r) asm volatile("" : "+r"(P.kb[r]));
+    constexpr unsigned step = kBlockPhilox * kTailMakers;
+    const float *end = ring + kTailRing * kNoiseBlock;
+    float *block = ring + rank * kNoiseBlock;
+    int to_go = round - rank;                        // blocks from this one to the round's end
+    for (int i = -2; kTailChunk * i < round; ++i) {   // makes chunk i + 2 while chunk i is used
+        if (to_go > 0) {
+#pragma unroll
+            for (int h = 0; h < kBlockPhilox; ++h) {
+                const uint4 x = philox_lane_block(P, lo, static_cast<unsigned>(h));
+                float2 rr;
+                float4 tg;
+                bm_pair_f32(x.x, x.y, bmc, rr.x, tg.x, tg.y);
+                bm_pair_f32(x.z, x.w, bmc, rr.y, tg.z, tg.w);
+                noise_store(block, lane, h, rr, tg);
+            }
+        }
+        to_go -= kTailMakers;
+        block += kTailChunk * kNoiseBlock;
+        if (block >= end) block -= kTailRing * kNoiseBlock;
+        lo += step;
+        if (__any_sync(kFull, lo < step)) {   // 2^32-block carry: new fixed words
+            if (lo < step) {
+                ++hi;
+                PhiloxLane Q;
+                philox_lane_init(Q, key0, key1, hi, gid_lo, gid_hi);
+                P.m0 = Q.m0;
+                P.x1m = Q.x1m;
+                P.z1m = Q.z1m;
+                P.z2m = Q.z2m;
+            }
+        }
+        if (i == -2) continue;   // the first barrier follows the second chunk
+        group_barrier(group);
+        if (i >= 0 && tail_sh.stop[i & 1][group]) break;
+    }
+}
+static_assert(kTailChunk == kTailMakers, "a noise warp makes one block of each chunk");
+
+// Runs the CTA's trajectories, `groups` groups of them in `lanes`, at most `blocks` blocks of
+// each, to the end of the launch (CTA-collective).
+__device__ __noinline__ void tail_run(const EngineDev &E, int *held, int groups, unsigned blocks) {
+    TailShared &sh = tail_sh;
+    TailLane *lanes = tail_lanes();
+    const int warp = static_cast<int>(threadIdx.x >> 5), lane = threadIdx.x & 31;
+    const int warps = static_cast<int>(blockDim.x >> 5);
+    const unsigned gtid = blockIdx.x * blockDim.x + threadIdx.x;
+    unsigned most = kRoundBlocks;   // doubled after each round that needed no packing
+    while (blocks > 0 && groups > 0) {
+        // Roles.  Euler: warp 4 g integrates group g (scheduler 0), the warps of the other
+        // schedulers make noise, the m-th of them for group m mod groups.  A Heun step's two sines
+        // take ~17 cycles of a scheduler: warp 2 g integrates (schedulers 0 and 2), the odd warps
+        // make noise and then the even ones that are left (four groups: 44 -> 33 ns per step).
+        bool heun = false;
+        for (int g = 0; g < groups; ++g) heun |= (sh.kind[g] & 2) != 0;
+        const int spread = heun ? 2 : 4;
+        const bool integrates = warp % spread == 0 && warp / spread < groups;
+        int m;
+        if (!heun) m = (warp & 3) == 0 ? 3 * kTailGroupsMax : (warp >> 2) * 3 + (warp & 3) - 1;
+        else m = (warp & 1) ? warp >> 1 : (warps >> 1) + (warp >> 1) - groups;
+        const int group = integrates ? warp / spread : m % groups;
+        const int rank = m / groups;
+        const int round = blocks < most ? static_cast<int>(blocks) : static_cast<int>(most);
+        if (integrates) {
+            switch (sh.kind[group]) {
+#define FPT_KIND_CASE(M_, H_, R_) \
+    case kind_of(M_, H_, R_): tail_integrate<M_, H_, R_>(E, group, round); break;
+            FPT_KIND_CASE(kUnder, kEuler, kConstBias)
+            FPT_KIND_CASE(kOver, kEuler, kConstBias)
+            FPT_KIND_CASE(kUnder, kHeun, kConstBias)
+            FPT_KIND_CASE(kOver, kHeun, kConstBias)
+            FPT_KIND_CASE(kUnder, kEuler, kRamp)
+            FPT_KIND_CASE(kOver, kEuler, kRamp)
+            FPT_KIND_CASE(kUnder, kHeun, kRamp)
+#undef FPT_KIND_CASE
+            default: tail_integrate<kOver, kHeun, kRamp>(E, group, round); break;
+            }
+        } else if (rank < kTailMakers) {
+            tail_noise(E, group, rank, round);
+        }
+        blocks -= static_cast<unsigned>(round);
+        __syncthreads();
+        if (warp < groups) {   // publish the round's results
+            TailLane &T = lanes[32 * warp + lane];
+            const bool fin = T.slot >= 0 && T.fin != kTailRuns;
+            emit_warp(E, held, fin, T.slot, (static_cast<unsigned long long>(T.gid_hi) << 32) | T.gid_lo,
+                      T.fin == kTailEscaped, (static_cast<unsigned long long>(T.c_hi) << 32) | T.c_lo);
+            if (fin) T.slot = -1;
+        }
+        int fewer = 0;
+        for (int g = 0, n = 0; g < groups; ++g) {
+            n += sh.alive[g];
+            if (g + 1 == groups || sh.kind[g + 1] != sh.kind[g]) {
+                fewer += (n + 31) >> 5;
+                n = 0;
+            }
+        }
+        __syncthreads();
+        if (fewer == groups) {
+            most *= 2u;
+            continue;
+        }
+        most = kRoundBlocks;
+        if (warp == 0) {   // close the gaps: entries only move down, past what has been read
+            int to = 0;    // next place
+            for (int g = 0; g < groups; ++g) {
+                const int k = sh.kind[g];
+                if (g > 0 && k != sh.kind[g - 1]) {   // a new kind starts a new group
+                    const int pad = (32 - (to & 31)) & 31;
+                    if (lane < pad) lanes[to + lane].slot = -1;
+                    to += pad;
+                }
+                const TailLane T = lanes[32 * g + lane];
+                const unsigned m = __ballot_sync(kFull, T.slot >= 0);
+                __syncwarp();
+                if (T.slot >= 0) lanes[to + __popc(m & ((1u << lane) - 1u))] = T;
+                __syncwarp();
+                const int first = (to + 31) >> 5, last = (to + __popc(m) + 31) >> 5;   // groups this one begins
+                if (lane == 0)
+                    for (int q = first; q < last; ++q) sh.count[q] = k;   // kinds of the new groups
+                to += __popc(m);
+            }
+            const int pad = (32 - (to & 31)) & 31;
+            if (lane < pad) lanes[to + lane].slot = -1;
+            __syncwarp();
+            if (lane < fewer) sh.kind[lane] = sh.count[lane];
+        }
+        groups = fewer;
+        __syncthreads();
+    }
+    // back into the lane state: group g in warp g
+    Lane L;
+    set_idle(L);
+    if (warp < groups) {
+        const TailLane T = lanes[32 * warp + lane];
+        if (T.slot >= 0) resume_from(L, E, T.slot, T);
+    }
+    store_lane(E, gtid, L);
+    if (lane == 0) E.warp_kind[gtid >> 5] = warp < groups ? sh.kind[warp] : -1;
+}
+
 template <int T>
-__global__ void __launch_bounds__(T == 1 ? 640 : 256, 1) engine_chunk_kernel(EngineDev E) {
+__global__ void __launch_bounds__(T == 1 ? 640 : 256, 1) engine_chunk_kernel(const __grid_constant__ EngineDev E) {
     const unsigned nthreads = gridDim.x * blockDim.x;
     const unsigned gtid = blockIdx.x * blockDim.x + threadIdx.x;
     const unsigned warp = gtid >> 5;
@@ -631,8 +1110,12 @@ __global__ void __launch_bounds__(T == 1 ? 640 : 256, 1) engine_chunk_kernel(Eng
     __shared__ int sh_res_slot[32], sh_res_cnt[32], sh_started[32];   // a CTA has at most 32 warps
     __shared__ unsigned long long sh_res_base[32];
     __shared__ int sh_pool;
-    __shared__ unsigned sh_chunk;
-    const CtaView V{sh_ok, sh_held, sh_budget, sh_res_slot, sh_res_cnt, sh_res_base, sh_started, &sh_pool};
+    __shared__ unsigned sh_chunk, sh_share;
+    __shared__ int sh_warp_act[32], sh_warp_knd[32], sh_tail, sh_done;
+    // while caps are enforced the lanes that idle are meant to
+    const int tail_groups = *E.strict != 0 ? 0 : tail_groups_of(T, static_cast<int>(blockDim.x >> 5));
+    const CtaView V{sh_ok, sh_held, sh_budget, sh_res_slot, sh_res_cnt, sh_res_base, sh_started, &sh_pool,
+                    sh_warp_act, sh_warp_knd, &sh_share, &sh_tail, tail_groups};
     for (int s = threadIdx.x; s < E.max_requests; s += blockDim.x) {
         sh_ok[s] = 0u;
         sh_held[s] = 0;
@@ -640,15 +1123,20 @@ __global__ void __launch_bounds__(T == 1 ? 640 : 256, 1) engine_chunk_kernel(Eng
     }
     if (threadIdx.x == 0) {
         sh_pool = 0;
+        sh_tail = 0;
+        sh_done = 0;
         // blocks per warp of this launch: the engine's full launch or a shorter one it chose
         const unsigned c = static_cast<unsigned>(*E.chunk_now);
         sh_chunk = c == 0u || c > E.chunk_blocks ? E.chunk_blocks : c;
+        sh_share = sh_chunk - sh_chunk / kPoolDiv;
     }
     if (threadIdx.x < 32) {
         sh_res_slot[threadIdx.x] = -1;
         sh_res_cnt[threadIdx.x] = 0;
         sh_res_base[threadIdx.x] = 0ull;
         sh_started[threadIdx.x] = 0;
+        sh_warp_act[threadIdx.x] = 0;
+        sh_warp_knd[threadIdx.x] = 0;
     }
     __syncthreads();
     {
@@ -683,19 +1171,7 @@ __global__ void __launch_bounds__(T == 1 ? 640 : 256, 1) engine_chunk_kernel(Eng
             set_idle(L[t]);
             continue;
         }
-        const SlotDev *S = E.slots + s;
-        L[t].slot = s;
-        L[t].r = E.lanes.r[i];
-        L[t].v = E.lanes.v[i];
-        L[t].hb = E.lanes.hb[i];
-        L[t].w = E.lanes.w[i];
-        L[t].c_lo = E.lanes.c_lo[i];
-        L[t].c_hi = E.lanes.c_hi[i];
-        L[t].gid_lo = E.lanes.gid_lo[i];
-        L[t].gid_hi = E.lanes.gid_hi[i];
-        L[t].esc = -1;
-        load_consts(L[t], S);
-        set_progress(L[t], S);
+        load_lane(L[t], E, i, s);
         atomicAdd(&sh_held[s], 1);
         ++n_active;
     }
@@ -713,31 +1189,94 @@ __global__ void __launch_bounds__(T == 1 ? 640 : 256, 1) engine_chunk_kernel(Eng
     // now, so a CTA whose warps are partly idle (fewer trajectories than lanes) gives its busy
     // warps as many blocks as a full CTA does, and all CTAs end together.
     if (lane == 0 && kind >= 0) atomicAdd(&sh_pool, static_cast<int>(sh_chunk / kPoolDiv));
+    {
+        const unsigned m = __ballot_sync(kFull, n_active > 0);
+        if (lane == 0) {
+            sh_warp_act[threadIdx.x >> 5] = __popc(m);
+            sh_warp_knd[threadIdx.x >> 5] = kind < 0 ? 0 : kind;
+        }
+    }
     __syncthreads();
-    unsigned limit = sh_chunk - sh_chunk / kPoolDiv;
-    while (b < limit || grant(V, limit)) {
-        if (kind < 0) {
-            kind = seek_work(L, E, V, n_active, cursor, b);
-            if (kind < 0) break;
-        }
-        switch (kind) {
+    if (T == 1 && threadIdx.x < 32 && tail_groups > 0) {
+        // dry from the start?  The queue heads as they are after this CTA's first claims.
+        for (int k = 0; k < kNumKinds; ++k)
+            for (int j = lane; j < E.act_count[k]; j += 32) {
+                const int s = E.act_list[k * E.max_requests + j];
+                if ((sh_ok[s] & 1u) && vload(E.ctl[s].head) >= E.slots[s].n_traj) atomicAnd(&sh_ok[s], ~1u);
+            }
+        __syncwarp();
+        look_dry(L, E, V, kind < 0 ? 0 : kind);
+    }
+    unsigned limit = 0;
+    for (bool again = true; again;) {   // again: the call to the last trajectories came too early
+        again = false;
+        while (b < limit || more(V, limit)) {
+            if (kind < 0) {
+                kind = seek_work(L, E, V, n_active, cursor, b);
+                if (kind < 0) break;
+                look_dry(L, E, V, kind);
+            }
+            switch (kind) {
 #define FPT_KIND_CASE(M_, H_, R_)                                                              \
-    case kind_of(M_, H_, R_):                                                                \
-        b = run_blocks<M_, H_, R_, T>(L, E, V, b, n_active, cursor, useful, n_esc, n_cens, limit); \
-        break;
-        FPT_KIND_CASE(kUnder, kEuler, kConstBias)
-        FPT_KIND_CASE(kOver, kEuler, kConstBias)
-        FPT_KIND_CASE(kUnder, kHeun, kConstBias)
-        FPT_KIND_CASE(kOver, kHeun, kConstBias)
-        FPT_KIND_CASE(kUnder, kEuler, kRamp)
-        FPT_KIND_CASE(kOver, kEuler, kRamp)
-        FPT_KIND_CASE(kUnder, kHeun, kRamp)
-        default:
-            b = run_blocks<kOver, kHeun, kRamp, T>(L, E, V, b, n_active, cursor, useful, n_esc, n_cens, limit);
+        case kind_of(M_, H_, R_):                                                                \
+            b = run_blocks<M_, H_, R_, T>(L, E, V, b, n_active, cursor, useful, n_esc, n_cens, limit); \
             break;
+            FPT_KIND_CASE(kUnder, kEuler, kConstBias)
+            FPT_KIND_CASE(kOver, kEuler, kConstBias)
+            FPT_KIND_CASE(kUnder, kHeun, kConstBias)
+            FPT_KIND_CASE(kOver, kHeun, kConstBias)
+            FPT_KIND_CASE(kUnder, kEuler, kRamp)
+            FPT_KIND_CASE(kOver, kEuler, kRamp)
+            FPT_KIND_CASE(kUnder, kHeun, kRamp)
+            default:
+                b = run_blocks<kOver, kHeun, kRamp, T>(L, E, V, b, n_active, cursor, useful, n_esc, n_cens, limit);
+                break;
 #undef FPT_KIND_CASE
+            }
+            if (!__any_sync(kFull, n_active > 0)) kind = -1;
         }
-        if (!__any_sync(kFull, n_active > 0)) kind = -1;
+        if constexpr (T == 1) {
+            if (tail_groups > 0) {
+                // the blocks left in this launch, after the furthest of the warps with trajectories
+                if (lane == 0 && kind >= 0) atomicMax(&sh_done, static_cast<int>(b));
+                __syncthreads();
+                if (sh_tail != 0) {
+                    int base, at;
+                    const int groups = tail_count(L, tail_sh.count, kind, base, at);
+                    if (groups <= tail_groups) {
+                        TailLane *lanes = tail_lanes();
+                        for (int i = threadIdx.x; i < 32 * groups; i += blockDim.x) lanes[i].slot = -1;
+                        __syncthreads();
+                        const unsigned have = __ballot_sync(kFull, L[0].slot >= 0);
+                        if (L[0].slot >= 0) {
+                            TailLane &P = lanes[32 * at + base + __popc(have & ((1u << lane) - 1u))];
+                            P.r = L[0].r;
+                            P.v = L[0].v;
+                            P.w = L[0].w;
+                            P.slot = L[0].slot;
+                            P.c_lo = L[0].c_lo;
+                            P.c_hi = L[0].c_hi;
+                            P.gid_lo = L[0].gid_lo;
+                            P.gid_hi = L[0].gid_hi;
+                            P.fin = kTailRuns;
+                        }
+                        if (threadIdx.x == 0)
+                            for (int k = 0, g = 0; k < kNumKinds; ++k)
+                                for (int n = tail_sh.count[k]; n > 0; n -= 32) tail_sh.kind[g++] = k;
+                        if (lane == 0) E.warp_cursor[warp] = cursor;
+                        add_counters(E, useful, n_esc, n_cens);
+                        const unsigned done = static_cast<unsigned>(sh_done);
+                        __syncthreads();
+                        tail_run(E, sh_held, groups, sh_chunk > done ? sh_chunk - done : 0u);
+                        return;
+                    }
+                    __syncthreads();   // a warp found more work after the call: go on as before
+                    if (threadIdx.x == 0) sh_tail = 0;
+                    __syncthreads();
+                    again = true;
+                }
+            }
+        }
     }
     // Preemption: a whole warp of this kind may be asked to vacate (so it can switch kind),
     // or single lanes of requests above their share to suspend.  Suspended state goes to the
@@ -805,35 +1344,12 @@ __global__ void __launch_bounds__(T == 1 ? 640 : 256, 1) engine_chunk_kernel(Eng
     }
     if (!__any_sync(kFull, n_active > 0)) kind = -1;
 #pragma unroll
-    for (int t = 0; t < T; ++t) {
-        const unsigned i = t * nthreads + gtid;
-        if (!checked(E, i < E.n_lanes, kChkLane)) continue;
-        E.lanes.slot[i] = L[t].slot;
-        if (L[t].slot < 0) continue;
-        E.lanes.r[i] = L[t].r;
-        E.lanes.v[i] = L[t].v;
-        E.lanes.hb[i] = L[t].hb;
-        E.lanes.w[i] = L[t].w;
-        E.lanes.c_lo[i] = L[t].c_lo;
-        E.lanes.c_hi[i] = L[t].c_hi;
-        E.lanes.gid_lo[i] = L[t].gid_lo;
-        E.lanes.gid_hi[i] = L[t].gid_hi;
-    }
+    for (int t = 0; t < T; ++t) store_lane(E, t * nthreads + gtid, L[t]);
     if (lane == 0) {
         E.warp_kind[warp] = kind;
         E.warp_cursor[warp] = cursor;
     }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        useful += __shfl_down_sync(kFull, useful, off);
-        n_esc += __shfl_down_sync(kFull, n_esc, off);
-        n_cens += __shfl_down_sync(kFull, n_cens, off);
-    }
-    if (lane == 0) {
-        if (useful) atomicAdd(&E.counters[kCntUseful], useful);
-        if (n_esc) atomicAdd(&E.counters[kCntEscapes], static_cast<unsigned long long>(n_esc));
-        if (n_cens) atomicAdd(&E.counters[kCntCensored], static_cast<unsigned long long>(n_cens));
-    }
+    add_counters(E, useful, n_esc, n_cens);
 }
 
 __device__ __forceinline__ double u128_to_d(unsigned long long lo, unsigned long long hi) {
@@ -902,8 +1418,12 @@ __global__ void engine_scan_kernel(EngineDev E) {
 
 cudaError_t launch_engine_chunk(const EngineDev &E, int T, unsigned grid, unsigned block,
                                 cudaStream_t s) {
-    if (T == 1) engine_chunk_kernel<1><<<grid, block, 0, s>>>(E);
-    else engine_chunk_kernel<2><<<grid, block, 0, s>>>(E);
+    if (T == 1) {
+        const size_t shared = tail_shared_bytes(static_cast<int>(block / 32));
+        engine_chunk_kernel<1><<<grid, block, shared, s>>>(E);
+    } else {
+        engine_chunk_kernel<2><<<grid, block, 0, s>>>(E);
+    }
     return cudaGetLastError();
 }
 
@@ -915,9 +1435,14 @@ cudaError_t launch_engine_scan(const EngineDev &E, cudaStream_t s) {
 }
 
 cudaError_t engine_chunk_occupancy(int T, int block, int *blocks_per_sm) {
-    if (T == 1)
-        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, engine_chunk_kernel<1>,
-                                                             block, 0);
+    if (T == 1) {
+        // every engine asks before its first launch, so the kernel's shared-memory limit is set
+        const cudaError_t e = cudaFuncSetAttribute(engine_chunk_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   static_cast<int>(tail_shared_bytes(640 / 32)));
+        if (e != cudaSuccess) return e;
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, engine_chunk_kernel<1>, block,
+                                                             tail_shared_bytes(block / 32));
+    }
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, engine_chunk_kernel<2>,
                                                          block, 0);
 }

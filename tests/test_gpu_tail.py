@@ -1,0 +1,66 @@
+"""The engine's last trajectories of a CTA (GPU): groups of an integrating warp and noise warps must
+give exactly the escape steps of the plain FP32 kernel, for counts around a group and around what
+the groups take on, launch lengths around a round and a chunk of noise, CTA sizes with one to five
+groups and none, every kind of step, and several kinds in one engine."""
+import numpy as np
+import pytest
+
+import workloads
+
+pytestmark = pytest.mark.gpu
+
+OVER = workloads.scaled(workloads.overdamped_sweep(n_traj=1)[11], dt=0.01, max_steps=10**6)
+UNDER = workloads.scaled(workloads.plain_constant_tilt(), D=0.08, dt=0.02, precision="fp32",
+                         max_steps=20011)
+RAMP = workloads.scaled(workloads.ramp_sweep(n_traj=1, rates=(2e-3,))[0])
+KINDS = [OVER, UNDER, RAMP, workloads.scaled(OVER, nu=1e-3), workloads.scaled(OVER, integrator="heun"),
+         workloads.scaled(UNDER, integrator="heun", dt=0.05), workloads.scaled(RAMP, integrator="heun"),
+         workloads.scaled(OVER, nu=1e-3, integrator="heun")]
+
+
+def _run(reqs, **kw):
+    import paper_1802_05065_gb300 as m
+    out = []
+    with m.Engine(0, **kw) as eng:
+        ids = [eng.submit(m.params_from(d, keep_per_traj=1), n, s) for d, n, s in reqs]
+        for rid, (d, n, s) in zip(ids, reqs):
+            r = eng.wait(rid, 300.0)
+            k = eng.per_traj_steps(rid, n)
+            h, u, o = eng.histogram(rid, d["hist_bins"])
+            assert r.n_used == n and sum(h) + u + o == (k >= 0).sum() == r.n_escaped
+            out.append(k)
+        assert eng.counters()["useful_steps"] == sum(
+            int(np.where(k >= 0, k, d["max_steps"]).sum()) for k, (d, _, _) in zip(out, reqs))
+    return out
+
+
+def _plain(d, n, s):
+    from paper_1802_05065_gb300 import api
+    return api.run_plain(d, n, s).cpu().numpy()
+
+
+@pytest.mark.parametrize("d", KINDS, ids=lambda d: f"{d['model']}-{d['integrator']}-{d['nu']:g}")
+@pytest.mark.parametrize("n", [1, 33, 152 * 32 * 4 + 17])
+def test_every_kind(d, n):
+    [k] = _run([(d, n, 90 + n)], chunk_steps=16384)
+    assert (k == _plain(d, n, 90 + n)).all()
+
+
+@pytest.mark.parametrize("chunk", [16, 48, 64, 144, 4096, 4112, 65536])
+def test_launch_lengths(chunk):
+    n = 4099 if chunk < 1000 else 152 * 160
+    d = workloads.scaled(OVER, max_steps=2000) if chunk < 1000 else OVER
+    [k] = _run([(d, n, 7)], chunk_steps=chunk)
+    assert (k == _plain(d, n, 7)).all()
+
+
+@pytest.mark.parametrize("threads", [128, 256, 288, 320, 416, 512, 640])
+def test_cta_sizes(threads):
+    [k] = _run([(OVER, 30011, 8)], chunk_steps=8192, threads_per_block=threads)
+    assert (k == _plain(OVER, 30011, 8)).all()
+
+
+def test_kinds_mixed():
+    reqs = [(d, 700 + 301 * i, 50 + i) for i, d in enumerate(KINDS)]
+    for k, (d, n, s) in zip(_run(reqs, chunk_steps=4096), reqs):
+        assert (k == _plain(d, n, s)).all()
