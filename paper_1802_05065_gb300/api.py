@@ -36,14 +36,13 @@ def reduce(d: dict, steps, **over):
     """Exact sums, moments and histogram of device escape steps (int64 tensor)."""
     torch = _torch()
     p = _lib.params_from(d, **over)
-    sums = torch.zeros(8, dtype=torch.int64, device=steps.device)
-    hist = torch.zeros(p.hist_bins, dtype=torch.int64, device=steps.device)
-    _lib.reduce_steps(p, steps.data_ptr(), steps.numel(), sums.data_ptr(), hist.data_ptr(),
+    out = torch.zeros(8 + p.hist_bins, dtype=torch.int64, device=steps.device)   # sums, histogram
+    _lib.reduce_steps(p, steps.data_ptr(), steps.numel(), out.data_ptr(), out.data_ptr() + 64,
                       current_stream(steps.device))
-    host = sums.cpu().numpy().view(np.uint64)
-    s = _lib.Sums(*[int(v) for v in host])
+    host = out.cpu().numpy()
+    s = _lib.Sums(*[int(v) for v in host[:8].view(np.uint64)])
     res = _lib.sums_finish(p, s)
-    return res, hist.cpu().numpy().view(np.uint64).astype(np.int64), s
+    return res, host[8:].copy(), s
 
 
 def philox_words(seed: int, traj: int, block0: int, nblocks: int, device=None) -> np.ndarray:

@@ -97,6 +97,35 @@ bool decode(const fpt_params *p, Decoded *d, std::string *err) {
     return true;
 }
 
+BinMap bin_map(const Decoded &d) {
+    BinMap m{0, UINT64_MAX, 0, 0, 0, 0, 0};
+    const double slope = d.out_b * d.hist_inv_w;   // bins per step
+    const double n = d.hist_bins;
+    if (!(slope > 0) || !(slope < 1) || !finite(d.hist_inv_w)) return m;
+    // steps where x reaches lo and hi (real numbers)
+    const double kl = (d.hist_lo - d.out_a) / d.out_b, kh = (d.hist_hi - d.out_a) / d.out_b;
+    if (!finite(kl) || !finite(kh) || !(kh > 1) || kh > 4503599627370496.0) return m;   // 2^52
+    // Off by, in bins: the formula's rounding, and kl's and kh's -- x and x - lo are each within
+    // 2^-52 of magnitudes up to |out_a| + |lo| + 2 |hi|, the rest is relative; the slope's double
+    // over the range; four units of the map's last place.
+    const double mag = std::fabs(d.out_a) + std::fabs(d.hist_lo) + 2 * std::fabs(d.hist_hi);
+    const double eps = std::ldexp(16.0, -52) * (mag * d.hist_inv_w + n) + std::ldexp(4.0, -32);
+    if (!(eps < 1.0 / 64)) return m;   // the formula would take too many steps anyway
+    const double margin = 2 * eps / slope + 2;   // steps that keep t more than eps from an end
+    m.k_under = kl > margin ? static_cast<uint64_t>(std::floor(kl - margin)) : 0;
+    m.k_over = static_cast<uint64_t>(std::ceil(kh + margin));
+    const double first = kl + margin > 0 ? std::ceil(kl + margin) : 0.0;
+    double last = std::floor(kh - margin);
+    if (last > 4294967295.0) last = 4294967295.0;
+    if (!(last > first)) return m;
+    m.first = static_cast<uint32_t>(first);
+    m.span = static_cast<uint32_t>(last - first);
+    m.slope = static_cast<uint64_t>(std::ldexp(slope, 64));
+    m.t_first = static_cast<uint64_t>(std::ldexp((d.out_a + d.out_b * first - d.hist_lo) * d.hist_inv_w, 32));
+    m.eps = static_cast<uint32_t>(std::ceil(std::ldexp(eps, 32)));
+    return m;
+}
+
 // 128-bit helpers (GCC/Clang on x86-64 and aarch64).
 using u128 = unsigned __int128;
 using i128 = __int128;

@@ -14,10 +14,12 @@
 
 #include <cstdint>
 
+#if !defined(FPT_HD)
 #if defined(__CUDACC__)
 #define FPT_HD __host__ __device__
 #else
 #define FPT_HD
+#endif
 #endif
 
 namespace fpt {
