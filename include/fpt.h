@@ -251,17 +251,11 @@ const char *fpt_status_string(fpt_status s);
  * theirs finishes, all in ONE launch that runs until every trajectory has finished, and calls
  * no cudaMalloc / cudaFree or allocating library routine.
  *
- * Scratch: a fixed 8 MiB __device__ array inside the library (every GPU that loads the library
- * holds it until the process exits): a queue head, a finished-CTA counter and one record of
- * partial sums and per-bin counts per CTA.  With many histogram bins the launch uses as many
- * CTAs as have room for their record (fewer CTAs, same result); hist_bins is limited to 10240
- * (the per-CTA histogram lives in shared memory) and n_traj to 2^32 - 1 (32-bit per-CTA bin
- * counts); larger requests are rejected with FPT_EINVAL and a message giving the limit.  The
- * first call on each device (and the first after that device's context changed, e.g. after
- * cudaDeviceReset) looks up the array's device address (cudaGetSymbolAddress) with that device
- * current; make that first call before any stream capture.  Every call shares the array: the
- * header is cleared on `stream` before each launch, and calls that overlap on the GPU (other
- * streams, other threads) race on it.
+ * Scratch: none in device memory.  Each CTA keeps the queue of its contiguous id range, its exact
+ * sums and its histogram in shared memory and adds them to the outputs when its range is done, so
+ * calls on other streams and threads may overlap, also with the same output buffers.  hist_bins is
+ * limited to 10240 (the per-CTA histogram lives in shared memory) and n_traj to 2^32 - 1 (32-bit
+ * per-CTA bin counts); larger requests are rejected with FPT_EINVAL and a message giving the limit.
  *
  * Arguments: params as for the engine but stop_rse must be 0; trajectories params->traj_offset
  * .. +n_traj-1 of `seed`.  d_steps (device, n_traj int64, may be NULL) receives each escape step

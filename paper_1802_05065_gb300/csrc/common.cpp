@@ -7,6 +7,7 @@
 #include <cstring>
 #include <string>
 
+#include "engine_dev.h"
 #include "internal.h"
 
 namespace fpt {
@@ -95,6 +96,39 @@ bool decode(const fpt_params *p, Decoded *d, std::string *err) {
     d->w0 = static_cast<int32_t>(w0);
     d->eb0_f = static_cast<float>(d->th - two_pi * w0);
     return true;
+}
+
+void slot_constants(const Decoded &d, uint64_t seed, uint64_t traj_offset, SlotDev *slot) {
+    SlotDev &S = *slot;
+    S.dt = d.dt_f;
+    S.A = d.A_f;
+    S.amp = d.amp_f;
+    S.bmc = d.bmc_f;
+    S.nudt = d.nudt_f;
+    S.v0 = d.v0_f;
+    S.r0 = d.r0_f;
+    S.eb0 = d.eb0_f;
+    S.w0 = d.w0;
+    S.kind = d.kind;
+    S.key0 = static_cast<uint32_t>(seed);
+    S.key1 = static_cast<uint32_t>(seed >> 32);
+    S.traj_offset = traj_offset;
+    S.max_steps = d.max_steps;
+    S.nblocks = (d.max_steps + 3) / 4;
+    S.gamma0 = d.gamma0;
+    S.nudt_d = d.nudt;
+    // the bias base and event countdown of a trajectory at block 0, as the kernel's
+    // set_progress forms them (c = c_base = 0; the re-base and carry counts are whole)
+    S.gb0 = static_cast<float>(d.gamma0 + d.nudt * static_cast<double>(0ull));
+    uint64_t m = S.nblocks < kRebaseBlocks ? S.nblocks : kRebaseBlocks;
+    S.budget0 = static_cast<uint32_t>((m + kBlockPhilox - 1) / kBlockPhilox);
+    S.output = d.output;
+    S.hist_bins = d.hist_bins;
+    S.out_a = d.out_a;
+    S.out_b = d.out_b;
+    S.hist_lo = d.hist_lo;
+    S.hist_hi = d.hist_hi;
+    S.hist_inv_w = d.hist_inv_w;
 }
 
 BinMap bin_map(const Decoded &d) {

@@ -273,40 +273,8 @@ fpt_status admit(fpt_engine *e) {
         const Decoded &d = R.dec;
         SlotDev &S = e->h_slots[s];
         std::memset(&S, 0, sizeof(S));
-        S.dt = d.dt_f;
-        S.A = d.A_f;
-        S.amp = d.amp_f;
-        S.bmc = d.bmc_f;
-        S.nudt = d.nudt_f;
-        S.v0 = d.v0_f;
-        S.r0 = d.r0_f;
-        S.eb0 = d.eb0_f;
-        S.w0 = d.w0;
-        S.kind = d.kind;
-        S.key0 = static_cast<uint32_t>(R.seed);
-        S.key1 = static_cast<uint32_t>(R.seed >> 32);
-        S.traj_offset = R.params.traj_offset;
+        slot_constants(d, R.seed, R.params.traj_offset, &S);
         S.n_traj = R.n_traj;
-        S.max_steps = d.max_steps;
-        S.nblocks = (d.max_steps + 3) / 4;
-        S.gamma0 = d.gamma0;
-        S.nudt_d = d.nudt;
-        // the bias base and event countdown of a trajectory at block 0, as the kernel's
-        // set_progress forms them (c = c_base = 0; the re-base and carry counts are whole)
-        S.gb0 = static_cast<float>(d.gamma0 + d.nudt * static_cast<double>(0ull));
-        {
-            const uint64_t to_end = S.nblocks, to_base = kRebaseBlocks, to_carry = 0x100000000ull;
-            uint64_t m = to_end < to_base ? to_end : to_base;
-            m = m < to_carry ? m : to_carry;
-            S.budget0 = static_cast<uint32_t>((m + kBlockPhilox - 1) / kBlockPhilox);
-        }
-        S.output = d.output;
-        S.hist_bins = d.hist_bins;
-        S.out_a = d.out_a;
-        S.out_b = d.out_b;
-        S.hist_lo = d.hist_lo;
-        S.hist_hi = d.hist_hi;
-        S.hist_inv_w = d.hist_inv_w;
         S.stop_rse = R.params.stop_rse;
         S.stop_block = R.stop_block;
         S.n_idblocks = R.n_idblocks;

@@ -116,6 +116,14 @@ struct SlotDev {
     unsigned park_cap;
 };
 
+// A request's constants in its slot: step, Philox key, first id, budget, observable and histogram
+// range.
+struct Decoded;
+void slot_constants(const Decoded &d, uint64_t seed, uint64_t traj_offset, SlotDev *S);
+
+// Histogram bins fpt_run_noalloc keeps per CTA in shared memory.
+constexpr int kSoloMaxBins = 10240;
+
 struct SlotCtl {
     unsigned long long head;   // next trajectory index to hand out (may run past n_traj)
     int inflight;              // lanes integrating a trajectory of this request

@@ -208,7 +208,7 @@ __device__ __forceinline__ void emit_warp(const EngineDev &E, int *held, bool fi
         idx = gid - S->traj_offset;
         ib = static_cast<unsigned>(id_block_quot(idx, S->ib_magic, S->ib_shift));
         row = S->hist_per_block ? ib : static_cast<unsigned>(idx / kHistRowIds);
-        if (escaped) bin = hist_bin(S, k);
+        if (escaped && S->hist) bin = hist_bin(S, k);
         fin = checked(E, idx < S->n_traj, kChkTraj) && checked(E, ib < S->n_idblocks, kChkIdBlock) &&
               checked(E, row < S->hist_rows, kChkHistRow) &&
               checked(E, bin == -2 || (bin >= -1 && bin <= S->hist_bins), kChkBin);
@@ -702,6 +702,16 @@ constexpr int kNoiseFloats = 24;                              // per lane and bl
 constexpr int kNoiseBlock = 32 * kNoiseFloats;                // floats of one block of a group
 constexpr int kTailMinWarps = 8;
 
+// A request that runs without an engine (solo_kernel).
+constexpr int kSoloThreads = 640;
+struct SoloArgs {
+    SlotDev slot;                  // n_traj, acc and hist are each CTA's own
+    unsigned long long n;
+    fpt_sums *sums;                // accumulated into, may be null
+    unsigned long long *hist;      // accumulated into: nbins counts, 0 without
+    int nbins;
+};
+
 struct TailLane {      // a trajectory while it changes warps, or its result
     float r, v;
     int w, slot;
@@ -714,7 +724,7 @@ enum : int { kTailRuns = 0, kTailEscaped = 1, kTailCensored = 2 };
 __host__ __device__ constexpr int tail_groups_of(int T, int warps) {
     return T != 1 || warps < kTailMinWarps ? 0 : (warps / 4 < kTailGroupsMax ? warps / 4 : kTailGroupsMax);
 }
-constexpr size_t tail_shared_bytes(int warps) {
+__host__ __device__ constexpr size_t tail_shared_bytes(int warps) {
     return tail_groups_of(1, warps) == 0 ? 0 : static_cast<size_t>(tail_groups_of(1, warps)) * kTailRing * kNoiseBlock * 4 +
                                                kTailGroupsMax * 32 * sizeof(TailLane);
 }
@@ -781,6 +791,36 @@ __device__ __forceinline__ int tail_count(Lane (&L)[1], int (&count)[kNumKinds],
         if (k == kind) at = groups;
         groups += (count[k] + 31) >> 5;
     }
+    return groups;
+}
+
+// Packs the CTA's trajectories for tail_run (CTA-collective): their groups, or -1 with nothing
+// changed when they are more than the CTA can run.
+__device__ __forceinline__ int tail_pack(Lane (&L)[1], const CtaView &V, int kind) {
+    const int lane = threadIdx.x & 31;
+    int base, at;
+    const int groups = tail_count(L, tail_sh.count, kind, base, at);
+    if (groups > V.tail_groups) return -1;
+    TailLane *lanes = tail_lanes();
+    for (int i = threadIdx.x; i < 32 * groups; i += blockDim.x) lanes[i].slot = -1;
+    __syncthreads();
+    const unsigned have = __ballot_sync(kFull, L[0].slot >= 0);
+    if (L[0].slot >= 0) {
+        TailLane &P = lanes[32 * at + base + __popc(have & ((1u << lane) - 1u))];
+        P.r = L[0].r;
+        P.v = L[0].v;
+        P.w = L[0].w;
+        P.slot = L[0].slot;
+        P.c_lo = L[0].c_lo;
+        P.c_hi = L[0].c_hi;
+        P.gid_lo = L[0].gid_lo;
+        P.gid_hi = L[0].gid_hi;
+        P.fin = kTailRuns;
+    }
+    if (threadIdx.x == 0)
+        for (int k = 0, g = 0; k < kNumKinds; ++k)
+            for (int n = tail_sh.count[k]; n > 0; n -= 32) tail_sh.kind[g++] = k;
+    __syncthreads();
     return groups;
 }
 
@@ -995,9 +1035,11 @@ __device__ __forceinline__ void tail_noise(const EngineDev &E, int group, int ra
 }
 static_assert(kTailChunk == kTailMakers, "a noise warp makes one block of each chunk");
 
-// Runs the CTA's trajectories, `groups` groups of them in `lanes`, at most `blocks` blocks of
-// each, to the end of the launch (CTA-collective).
-__device__ __noinline__ void tail_run(const EngineDev &E, int *held, int groups, unsigned blocks) {
+// Runs the CTA's trajectories, `groups` packed groups of them, at most `blocks` blocks of each, to
+// the end of the launch (CTA-collective), and leaves the rest in the lane state if there is one.
+// K: the kind of every group, or -1.
+template <int K>
+__device__ __noinline__ void tail_run(const EngineDev &E, int *held, int groups, unsigned long long blocks) {
     TailShared &sh = tail_sh;
     TailLane *lanes = tail_lanes();
     const int warp = static_cast<int>(threadIdx.x >> 5), lane = threadIdx.x & 31;
@@ -1020,7 +1062,8 @@ __device__ __noinline__ void tail_run(const EngineDev &E, int *held, int groups,
         const int rank = m / groups;
         const int round = blocks < most ? static_cast<int>(blocks) : static_cast<int>(most);
         if (integrates) {
-            switch (sh.kind[group]) {
+            if constexpr (K >= 0) tail_integrate<(K & 1), ((K >> 1) & 1), (K >> 2)>(E, group, round);
+            else switch (sh.kind[group]) {
 #define FPT_KIND_CASE(M_, H_, R_) \
     case kind_of(M_, H_, R_): tail_integrate<M_, H_, R_>(E, group, round); break;
             FPT_KIND_CASE(kUnder, kEuler, kConstBias)
@@ -1086,6 +1129,7 @@ __device__ __noinline__ void tail_run(const EngineDev &E, int *held, int groups,
         groups = fewer;
         __syncthreads();
     }
+    if (!E.lanes.slot) return;
     // back into the lane state: group g in warp g
     Lane L;
     set_idle(L);
@@ -1241,33 +1285,12 @@ __global__ void __launch_bounds__(T == 1 ? 640 : 256, 1) engine_chunk_kernel(con
                 if (lane == 0 && kind >= 0) atomicMax(&sh_done, static_cast<int>(b));
                 __syncthreads();
                 if (sh_tail != 0) {
-                    int base, at;
-                    const int groups = tail_count(L, tail_sh.count, kind, base, at);
-                    if (groups <= tail_groups) {
-                        TailLane *lanes = tail_lanes();
-                        for (int i = threadIdx.x; i < 32 * groups; i += blockDim.x) lanes[i].slot = -1;
-                        __syncthreads();
-                        const unsigned have = __ballot_sync(kFull, L[0].slot >= 0);
-                        if (L[0].slot >= 0) {
-                            TailLane &P = lanes[32 * at + base + __popc(have & ((1u << lane) - 1u))];
-                            P.r = L[0].r;
-                            P.v = L[0].v;
-                            P.w = L[0].w;
-                            P.slot = L[0].slot;
-                            P.c_lo = L[0].c_lo;
-                            P.c_hi = L[0].c_hi;
-                            P.gid_lo = L[0].gid_lo;
-                            P.gid_hi = L[0].gid_hi;
-                            P.fin = kTailRuns;
-                        }
-                        if (threadIdx.x == 0)
-                            for (int k = 0, g = 0; k < kNumKinds; ++k)
-                                for (int n = tail_sh.count[k]; n > 0; n -= 32) tail_sh.kind[g++] = k;
+                    const int groups = tail_pack(L, V, kind);
+                    if (groups >= 0) {
                         if (lane == 0) E.warp_cursor[warp] = cursor;
                         add_counters(E, useful, n_esc, n_cens);
                         const unsigned done = static_cast<unsigned>(sh_done);
-                        __syncthreads();
-                        tail_run(E, sh_held, groups, sh_chunk > done ? sh_chunk - done : 0u);
+                        tail_run<-1>(E, sh_held, groups, sh_chunk > done ? sh_chunk - done : 0u);
                         return;
                     }
                     __syncthreads();   // a warp found more work after the call: go on as before
@@ -1367,6 +1390,118 @@ __device__ __forceinline__ void add_limbs(unsigned long long &lo, unsigned long 
     hi += ah + (lo < a ? 1ull : 0ull) + l2;
 }
 
+// ---- one request without an engine ------------------------------------------------------------
+// fpt_run_noalloc on the machinery above: each CTA is an engine of its own for a contiguous range of the ids, its slot,
+// queue and accumulators in shared memory, so a call needs no scratch in device memory and shares
+// nothing with other calls; it runs until its range is done and adds its exact sums and counts to
+// the caller's.  Ranges of equal size differ in length by a few percent, less than the last
+// trajectories take.  Against one event test per step, a full Philox per call and one queue for all
+// CTAs (256 threads each): 200 003 trajectories of 19 000 steps 16.8 -> 6.5 ms.
+template <int M, int H, int R>
+__global__ void __launch_bounds__(kSoloThreads, 1) solo_kernel(const __grid_constant__ SoloArgs a) {
+    const int warp = static_cast<int>(threadIdx.x >> 5), lane = threadIdx.x & 31;
+    constexpr int kind = kind_of(M, H, R);
+    __shared__ SlotDev slot;
+    __shared__ SlotCtl ctl;
+    __shared__ IdBlockAcc acc;
+    __shared__ EngineDev E;
+    __shared__ unsigned long long counters[kCntCount], res_base[32];
+    __shared__ unsigned ok, share;
+    __shared__ int held, budget, pool, tail, claim, zeros[kNumKinds], counts[kNumKinds];
+    __shared__ int res_slot[32], res_cnt[32], started[32], warp_act[32], warp_knd[32];
+    unsigned *hist = reinterpret_cast<unsigned *>(tail_mem + tail_shared_bytes(kSoloThreads / 32));
+    const CtaView V{&ok, &held, &budget, res_slot, res_cnt, res_base, started, &pool, warp_act, warp_knd, &share, &tail,
+                    tail_groups_of(1, kSoloThreads / 32)};
+    for (int b = threadIdx.x; b < a.nbins; b += blockDim.x) hist[b] = 0u;
+    if (threadIdx.x < 32) {
+        res_slot[threadIdx.x] = -1;
+        res_cnt[threadIdx.x] = started[threadIdx.x] = warp_act[threadIdx.x] = 0;
+        warp_knd[threadIdx.x] = kind;
+        res_base[threadIdx.x] = 0ull;
+    }
+    if (threadIdx.x < kNumKinds) {
+        zeros[threadIdx.x] = 0;
+        counts[threadIdx.x] = threadIdx.x == kind ? 1 : 0;
+    }
+    if (threadIdx.x == 0) {
+        const unsigned long long first = a.n * blockIdx.x / gridDim.x, end = a.n * (blockIdx.x + 1ull) / gridDim.x;
+        slot = a.slot;
+        slot.n_traj = end;
+        slot.acc = &acc;
+        slot.hist = a.nbins ? hist : nullptr;
+        ctl = SlotCtl{};
+        ctl.head = first;
+        ctl.state = kSlotActive;
+        acc = IdBlockAcc{};
+        for (int i = 0; i < kCntCount; ++i) counters[i] = 0ull;
+        E = EngineDev{};
+        E.slots = &slot;
+        E.ctl = &ctl;
+        E.strict = zeros;
+        E.claim_warps = &claim;
+        E.act_list = zeros;
+        E.act_count = counts;
+        E.counters = counters;
+        E.max_requests = 1;
+        E.n_lanes = gridDim.x * blockDim.x;
+        ok = first < end ? 1u : 0u;
+        held = budget = pool = tail = 0;
+        share = 0x80000000u;   // blocks before the warps meet in any case (they go on)
+        const unsigned long long warps = (end - first + 31) / 32;
+        claim = warps < kSoloThreads / 32 ? static_cast<int>(warps) : kSoloThreads / 32;
+    }
+    __syncthreads();
+    Lane L[1];
+    set_idle(L[0]);
+    int n_active = 0;
+    unsigned cursor = 0, n_esc = 0, n_cens = 0;
+    unsigned long long useful = 0;
+    refill(L, E, V, kind, n_active, cursor, 0u);
+    {
+        const unsigned m = __ballot_sync(kFull, n_active > 0);
+        if (lane == 0) warp_act[warp] = __popc(m);
+    }
+    __syncthreads();
+    if (warp == 0) {
+        if (lane == 0 && ctl.head >= slot.n_traj) ok = 0u;
+        __syncwarp();
+        look_dry(L, E, V, kind);
+    }
+    for (;;) {
+        unsigned b = 0, limit = 0;
+        if (__any_sync(kFull, n_active > 0))
+            run_blocks<M, H, R, 1>(L, E, V, b, n_active, cursor, useful, n_esc, n_cens, limit);
+        __syncthreads();
+        if (tail != 0) {
+            const int groups = tail_pack(L, V, kind);
+            if (groups >= 0) {
+                tail_run<kind>(E, &held, groups, ~0ull);
+                break;
+            }
+            __syncthreads();
+            if (threadIdx.x == 0) tail = 0;
+        }
+        if (!__syncthreads_or(n_active > 0)) break;
+    }
+    __syncthreads();
+    if (a.sums && threadIdx.x == 0) {
+        unsigned long long s1lo = 0, s1hi = 0, s2lo = 0, s2hi = 0;
+        add_limbs(s1lo, s1hi, acc.s1[0], acc.s1[1], 0ull);
+        add_limbs(s2lo, s2hi, acc.s2[0], acc.s2[1], acc.s2[2]);
+        unsigned long long *o = reinterpret_cast<unsigned long long *>(a.sums);
+        atomicAdd(&o[0], static_cast<unsigned long long>(acc.done));
+        if (acc.escaped) atomicAdd(&o[1], static_cast<unsigned long long>(acc.escaped));
+        const unsigned long long p1 = atomicAdd(&o[2], s1lo);
+        if (s1hi + (p1 + s1lo < p1 ? 1ull : 0ull)) atomicAdd(&o[3], s1hi + (p1 + s1lo < p1 ? 1ull : 0ull));
+        const unsigned long long p2 = atomicAdd(&o[4], s2lo);
+        if (s2hi + (p2 + s2lo < p2 ? 1ull : 0ull)) atomicAdd(&o[5], s2hi + (p2 + s2lo < p2 ? 1ull : 0ull));
+        if (acc.under) atomicAdd(&o[6], static_cast<unsigned long long>(acc.under));
+        if (acc.over) atomicAdd(&o[7], static_cast<unsigned long long>(acc.over));
+    }
+    for (int b = threadIdx.x; b < a.nbins; b += blockDim.x)
+        if (hist[b]) atomicAdd(&a.hist[b], static_cast<unsigned long long>(hist[b]));
+}
+
 // Fold completed id blocks, in id order, into each request's running sums; stop at the first
 // prefix meeting the relative-standard-error rule, or when every block is complete.
 __global__ void engine_scan_kernel(EngineDev E) {
@@ -1424,6 +1559,49 @@ cudaError_t launch_engine_chunk(const EngineDev &E, int T, unsigned grid, unsign
     } else {
         engine_chunk_kernel<2><<<grid, block, 0, s>>>(E);
     }
+    return cudaGetLastError();
+}
+
+cudaError_t launch_solo(const Decoded &d, uint64_t seed, uint64_t traj_offset, uint64_t n, int64_t *steps,
+                        fpt_sums *sums, unsigned long long *hist, cudaStream_t s) {
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    SoloArgs a{};
+    slot_constants(d, seed, traj_offset, &a.slot);
+    a.slot.n_traj = n;
+    a.slot.stop_block = 0xFFFFFFFFu;
+    a.slot.n_idblocks = 1;
+    id_block_magic(a.slot.stop_block, a.slot.ib_magic, a.slot.ib_shift);
+    a.slot.hist_per_block = 1;   // one row
+    a.slot.hist_rows = 1;
+    a.slot.per_traj = reinterpret_cast<long long *>(steps);
+    a.slot.park_cap = 1;
+    a.n = n;
+    a.sums = sums;
+    a.hist = hist;
+    a.nbins = hist ? d.hist_bins : 0;
+    void (*kernel)(SoloArgs) = nullptr;
+    switch (d.kind) {
+#define FPT_KIND_CASE(M_, H_, R_) \
+    case kind_of(M_, H_, R_): kernel = solo_kernel<M_, H_, R_>; break;
+    FPT_KIND_CASE(kUnder, kEuler, kConstBias)
+    FPT_KIND_CASE(kOver, kEuler, kConstBias)
+    FPT_KIND_CASE(kUnder, kHeun, kConstBias)
+    FPT_KIND_CASE(kOver, kHeun, kConstBias)
+    FPT_KIND_CASE(kUnder, kEuler, kRamp)
+    FPT_KIND_CASE(kOver, kEuler, kRamp)
+    FPT_KIND_CASE(kUnder, kHeun, kRamp)
+#undef FPT_KIND_CASE
+    default: kernel = solo_kernel<kOver, kHeun, kRamp>; break;
+    }
+    const size_t shared = tail_shared_bytes(kSoloThreads / 32) + static_cast<size_t>(a.nbins) * 4;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             static_cast<int>(tail_shared_bytes(kSoloThreads / 32) + kSoloMaxBins * 4));
+    if (e != cudaSuccess) return e;
+    const uint64_t warps = (n + 31) / 32;
+    kernel<<<static_cast<unsigned>(warps < static_cast<uint64_t>(sms) ? warps : sms), kSoloThreads, shared, s>>>(a);
     return cudaGetLastError();
 }
 

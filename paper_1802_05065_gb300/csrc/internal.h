@@ -80,6 +80,10 @@ struct PlainArgs {
     float dt_f, A_f, amp_f, bmc_f, nudt_f, v0_f, r0_f, eb0_f;
     int32_t w0;
 };
+// One FP32 request on the resident kernel's machinery, run to completion (engine_kernels.cu): escape
+// steps, sums and histogram each optional.  n < 2^32, hist_bins <= kSoloMaxBins with a histogram.
+cudaError_t launch_solo(const Decoded &d, uint64_t seed, uint64_t traj_offset, uint64_t n, int64_t *steps,
+                        fpt_sums *sums, unsigned long long *hist, cudaStream_t s);
 cudaError_t launch_plain_f64(const PlainArgs &a, cudaStream_t s);
 cudaError_t launch_plain_f32(const PlainArgs &a, cudaStream_t s);
 

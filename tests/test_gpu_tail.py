@@ -34,7 +34,7 @@ def _run(reqs, **kw):
     return out
 
 
-def _plain(d, n, s):
+def _plain(d, n, s):   # one trajectory per thread, no shared machinery
     from paper_1802_05065_gb300 import api
     return api.run_plain(d, n, s).cpu().numpy()
 
