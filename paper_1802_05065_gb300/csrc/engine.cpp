@@ -7,7 +7,7 @@
 //   2. the claimable-slot lists and fair-share caps are refreshed (pinned host -> device);
 //   3. one resident-kernel launch advances every lane by up to chunk_steps steps;
 //   4. the scan kernel folds completed id blocks and applies the stop rule;
-//   5. the per-slot status and counters come back to pinned host memory.
+//   5. the scan kernel writes the per-slot status and counters to pinned host memory.
 // Steps 2-5 are one CUDA graph.  Slots are reused only after no lane holds a trajectory of the
 // old request (its in-flight count has reached zero).
 //
@@ -39,7 +39,7 @@
 namespace fpt {
 cudaError_t launch_engine_chunk(const EngineDev &E, int T, unsigned grid, unsigned block,
                                 cudaStream_t s);
-cudaError_t launch_engine_scan(const EngineDev &E, cudaStream_t s);
+cudaError_t launch_engine_scan(const EngineDev &E, SlotCtl *h_ctl, unsigned long long *h_counters, cudaStream_t s);
 cudaError_t engine_chunk_occupancy(int T, int block, int *blocks_per_sm);
 }  // namespace fpt
 
@@ -131,11 +131,12 @@ size_t request_bytes(const fpt_params &p, uint64_t n_traj, uint32_t B, unsigned 
 // Host side of one in-flight iteration: the lists it uploads, the status it downloads, its
 // events and its graph.  Two alternate.
 struct IterIO {
+    int *lists = nullptr;                       // one pinned block, uploaded in one copy, of ...
     int *caps = nullptr, *act = nullptr, *act_count = nullptr;
     int *preempt = nullptr, *flags = nullptr;   // flags: vacate[kNumKinds], strict, claim_warps,
                                                 // blocks per warp of the launch
-    SlotCtl *ctl = nullptr;                     // status download target
-    unsigned long long *counters = nullptr;     // counters download target
+    SlotCtl *ctl = nullptr;                     // pinned: the scan kernel writes the status here
+    unsigned long long *counters = nullptr;     // and the counters here
     cudaEvent_t k0 = nullptr, k1 = nullptr;     // around the resident kernel
     cudaEvent_t done = nullptr;                 // after the downloads
     cudaGraph_t graph = nullptr;
@@ -146,6 +147,12 @@ struct IterIO {
 
 // Flags uploaded with each launch: vacate[kNumKinds], strict, claim_warps, blocks per warp.
 constexpr int kNumFlags = kNumKinds + 3;
+
+// The lists of a launch in their block (host and device alike): flags, claimable slots per kind,
+// caps, preemption orders, the claimable slots of each kind.
+constexpr int kListFlags = 0, kListCounts = 16, kListCaps = kListCounts + kNumKinds;
+static_assert(kNumFlags <= kListCounts, "flags fit in front of the counts");
+constexpr size_t list_ints(int maxr) { return kListCaps + static_cast<size_t>(maxr) * (2 + kNumKinds); }
 
 // Launches after its admission during which a request that fits in the lanes counts as young
 // (the launch length is then the engine's young_chunk_steps).
@@ -163,8 +170,7 @@ struct fpt_engine {
     // device
     SlotDev *d_slots = nullptr;
     SlotCtl *d_ctl = nullptr;
-    int *d_caps = nullptr, *d_act = nullptr, *d_act_count = nullptr;
-    int *d_preempt = nullptr, *d_vacate = nullptr, *d_strict = nullptr;
+    int *d_lists = nullptr;       // see list_ints
     void *d_lane_mem = nullptr;
     int *d_warp_kind = nullptr;
     unsigned *d_warp_cursor = nullptr;
@@ -448,22 +454,12 @@ fpt_status enqueue_iteration(fpt_engine *e, IterIO &B) {
         CK(cudaGraphLaunch(B.exec, e->stream));
         return FPT_OK;
     }
-    CK(cudaMemcpyAsync(e->d_caps, B.caps, e->maxr * sizeof(int), cudaMemcpyHostToDevice, e->stream));
-    CK(cudaMemcpyAsync(e->d_preempt, B.preempt, e->maxr * sizeof(int), cudaMemcpyHostToDevice, e->stream));
-    CK(cudaMemcpyAsync(e->d_vacate, B.flags, kNumFlags * sizeof(int), cudaMemcpyHostToDevice,
-                       e->stream));
-    CK(cudaMemcpyAsync(e->d_act, B.act, kNumKinds * e->maxr * sizeof(int), cudaMemcpyHostToDevice,
-                       e->stream));
-    CK(cudaMemcpyAsync(e->d_act_count, B.act_count, kNumKinds * sizeof(int), cudaMemcpyHostToDevice,
-                       e->stream));
+    CK(cudaMemcpyAsync(e->d_lists, B.lists, list_ints(e->maxr) * sizeof(int), cudaMemcpyHostToDevice, e->stream));
     const unsigned evflags = e->capturing ? cudaEventRecordExternal : cudaEventRecordDefault;
     CK(cudaEventRecordWithFlags(B.k0, e->stream, evflags));
     CK(launch_engine_chunk(e->dev, e->T, e->grid, e->block, e->stream));
     CK(cudaEventRecordWithFlags(B.k1, e->stream, evflags));
-    CK(launch_engine_scan(e->dev, e->stream));
-    CK(cudaMemcpyAsync(B.ctl, e->d_ctl, e->maxr * sizeof(SlotCtl), cudaMemcpyDeviceToHost, e->stream));
-    CK(cudaMemcpyAsync(B.counters, e->d_counters, kCntCount * sizeof(unsigned long long),
-                       cudaMemcpyDeviceToHost, e->stream));
+    CK(launch_engine_scan(e->dev, B.ctl, B.counters, e->stream));
     return FPT_OK;
 }
 
@@ -525,7 +521,8 @@ fpt_status complete_oldest(fpt_engine *e) {
     CK(cudaEventElapsedTime(&ms, B.k0, B.k1));
     {
         std::lock_guard<std::mutex> lk(e->mu);
-        std::memcpy(e->h_ctl, B.ctl, e->maxr * sizeof(SlotCtl));
+        for (int s = 0; s < e->maxr; ++s)
+            if (e->slot_req[s]) e->h_ctl[s] = B.ctl[s];
         std::memcpy(e->h_counters, B.counters, kCntCount * sizeof(unsigned long long));
         e->status_seq = B.seq;
         process_status(e);
@@ -636,11 +633,7 @@ void destroy_all(fpt_engine *e) {
     for (IterIO &B : e->iters) {
         if (B.exec) cudaGraphExecDestroy(B.exec);
         if (B.graph) cudaGraphDestroy(B.graph);
-        cudaFreeHost(B.caps);
-        cudaFreeHost(B.act);
-        cudaFreeHost(B.act_count);
-        cudaFreeHost(B.preempt);
-        cudaFreeHost(B.flags);
+        cudaFreeHost(B.lists);
         cudaFreeHost(B.ctl);
         cudaFreeHost(B.counters);
         if (B.k0) cudaEventDestroy(B.k0);
@@ -649,11 +642,7 @@ void destroy_all(fpt_engine *e) {
     }
     cudaFree(e->d_slots);
     cudaFree(e->d_ctl);
-    cudaFree(e->d_caps);
-    cudaFree(e->d_act);
-    cudaFree(e->d_act_count);
-    cudaFree(e->d_preempt);
-    cudaFree(e->d_vacate);
+    cudaFree(e->d_lists);
     cudaFree(e->d_lane_mem);
     cudaFree(e->d_warp_kind);
     cudaFree(e->d_warp_cursor);
@@ -713,13 +702,8 @@ fpt_status create_impl(const fpt_engine_config *cfg_in, fpt_engine *e) {
     const int R = e->maxr;
     CK(cudaMalloc(&e->d_slots, R * sizeof(SlotDev)));
     CK(cudaMalloc(&e->d_ctl, R * sizeof(SlotCtl)));
-    CK(cudaMalloc(&e->d_caps, R * sizeof(int)));
-    CK(cudaMalloc(&e->d_act, kNumKinds * R * sizeof(int)));
-    CK(cudaMalloc(&e->d_act_count, kNumKinds * sizeof(int)));
-    CK(cudaMalloc(&e->d_preempt, R * sizeof(int)));
-    CK(cudaMalloc(&e->d_vacate, kNumFlags * sizeof(int)));   // vacate[kNumKinds], strict, claim, chunk
-    CK(cudaMemsetAsync(e->d_preempt, 0, R * sizeof(int), e->stream));
-    CK(cudaMemsetAsync(e->d_vacate, 0, kNumFlags * sizeof(int), e->stream));
+    CK(cudaMalloc(&e->d_lists, list_ints(R) * sizeof(int)));
+    CK(cudaMemsetAsync(e->d_lists, 0, list_ints(R) * sizeof(int), e->stream));
     const size_t L = e->lanes;
     CK(cudaMalloc(&e->d_lane_mem, L * 4 * 10));
     const unsigned nwarps = static_cast<unsigned>(e->grid) * e->block / 32;
@@ -756,18 +740,15 @@ fpt_status create_impl(const fpt_engine_config *cfg_in, fpt_engine *e) {
     std::memset(e->h_ctl, 0, R * sizeof(SlotCtl));
     std::memset(e->h_counters, 0, kCntCount * sizeof(unsigned long long));
     for (IterIO &B : e->iters) {
-        CK(cudaMallocHost(&B.caps, R * sizeof(int)));
-        CK(cudaMallocHost(&B.act, kNumKinds * R * sizeof(int)));
-        CK(cudaMallocHost(&B.act_count, kNumKinds * sizeof(int)));
-        CK(cudaMallocHost(&B.preempt, R * sizeof(int)));
-        CK(cudaMallocHost(&B.flags, kNumFlags * sizeof(int)));
+        CK(cudaMallocHost(&B.lists, list_ints(R) * sizeof(int)));
+        std::memset(B.lists, 0, list_ints(R) * sizeof(int));
+        B.flags = B.lists + kListFlags;
+        B.act_count = B.lists + kListCounts;
+        B.caps = B.lists + kListCaps;
+        B.preempt = B.caps + R;
+        B.act = B.preempt + R;
         CK(cudaMallocHost(&B.ctl, R * sizeof(SlotCtl)));
         CK(cudaMallocHost(&B.counters, kCntCount * sizeof(unsigned long long)));
-        std::memset(B.caps, 0, R * sizeof(int));
-        std::memset(B.act, 0, kNumKinds * R * sizeof(int));
-        std::memset(B.act_count, 0, kNumKinds * sizeof(int));
-        std::memset(B.preempt, 0, R * sizeof(int));
-        std::memset(B.flags, 0, kNumFlags * sizeof(int));
         std::memset(B.ctl, 0, R * sizeof(SlotCtl));
         std::memset(B.counters, 0, kCntCount * sizeof(unsigned long long));
         CK(cudaEventCreate(&B.k0));
@@ -778,14 +759,15 @@ fpt_status create_impl(const fpt_engine_config *cfg_in, fpt_engine *e) {
     EngineDev &d = e->dev;
     d.slots = e->d_slots;
     d.ctl = e->d_ctl;
-    d.caps = e->d_caps;
-    d.act_list = e->d_act;
-    d.preempt = e->d_preempt;
-    d.vacate = e->d_vacate;
-    d.strict = e->d_vacate + kNumKinds;
-    d.claim_warps = e->d_vacate + kNumKinds + 1;
-    d.chunk_now = e->d_vacate + kNumKinds + 2;
-    d.act_count = e->d_act_count;
+    int *flags = e->d_lists + kListFlags;
+    d.vacate = flags;
+    d.strict = flags + kNumKinds;
+    d.claim_warps = flags + kNumKinds + 1;
+    d.chunk_now = flags + kNumKinds + 2;
+    d.act_count = e->d_lists + kListCounts;
+    d.caps = e->d_lists + kListCaps;
+    d.preempt = e->d_lists + kListCaps + R;
+    d.act_list = e->d_lists + kListCaps + 2 * R;
     d.warp_kind = e->d_warp_kind;
     d.warp_cursor = e->d_warp_cursor;
     d.counters = e->d_counters;

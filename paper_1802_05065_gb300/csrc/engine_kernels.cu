@@ -1,4 +1,5 @@
-// engine_kernels.cu -- the persistent batched FPT kernel and the completion scan.
+// engine_kernels.cu -- the persistent batched FPT kernel, the completion scan, and one request's
+// kernel without an engine.
 //
 // One launch ("chunk") advances the resident lanes by the launch's blocks of kBlockSteps steps
 // per warp on average (chunk_blocks, or fewer while a small request is new; Euler-Maruyama or
@@ -185,6 +186,8 @@ struct CtaView {
     unsigned *share;             // blocks of the launch every warp runs before it takes from the pool
     int *tail;                   // 1: the CTA's warps meet to run its last trajectories together
     int tail_groups;             // groups of 32 lanes the CTA can run that way (0: it never does)
+    const int *act_count;        // the launch's lists and flags, read once: claimable slots per kind,
+    const int *flags;            // {strict caps, warps of the CTA that claim}
 };
 
 // Publish the trajectories finishing in this warp at this block end (warp-collective: every lane
@@ -362,12 +365,12 @@ __device__ __forceinline__ int refill(Lane (&L)[T], const EngineDev &E, const Ct
         total += __popc(idle[t]);
     }
     if (total == 0) return 0;
-    if (static_cast<int>(threadIdx.x >> 5) >= *E.claim_warps) return total;   // spread scarce work
+    if (static_cast<int>(threadIdx.x >> 5) >= V.flags[1]) return total;   // spread scarce work
     if (!checked(E, kind >= 0 && kind < kNumKinds, kChkKind)) return total;
-    const int cnt = E.act_count[kind];
+    const int cnt = V.act_count[kind];
     if (cnt <= 0) return total;
     const int *list = E.act_list + kind * E.max_requests;
-    const bool capped = *E.strict != 0;
+    const bool capped = V.flags[0] != 0;
     const int wl = static_cast<int>(threadIdx.x >> 5);
     // A warp that holds a reservoir serves its request first, so the reservoir drains.
     __syncwarp();
@@ -534,7 +537,7 @@ __device__ __forceinline__ void look_dry(Lane (&L)[T], const EngineDev &E, const
         if (total == 0 || total + (kinds > 1 ? 31 * kinds : 0) > 32 * V.tail_groups) return;
         bool work = lane < warps && vload(V.res_cnt[lane]) > 0;
         for (int k = 0; k < kNumKinds; ++k)
-            for (int j = lane; j < E.act_count[k]; j += 32)
+            for (int j = lane; j < V.act_count[k]; j += 32)
                 work |= (vload(V.ok[E.act_list[k * E.max_requests + j]]) & 3u) != 0u;
         if (!__any_sync(kFull, work) && lane == 0) *V.tail = 1;
     }
@@ -1155,11 +1158,11 @@ __global__ void __launch_bounds__(T == 1 ? 640 : 256, 1) engine_chunk_kernel(con
     __shared__ unsigned long long sh_res_base[32];
     __shared__ int sh_pool;
     __shared__ unsigned sh_chunk, sh_share;
-    __shared__ int sh_warp_act[32], sh_warp_knd[32], sh_tail, sh_done;
+    __shared__ int sh_warp_act[32], sh_warp_knd[32], sh_tail, sh_done, sh_act_count[kNumKinds], sh_flags[2];
     // while caps are enforced the lanes that idle are meant to
     const int tail_groups = *E.strict != 0 ? 0 : tail_groups_of(T, static_cast<int>(blockDim.x >> 5));
     const CtaView V{sh_ok, sh_held, sh_budget, sh_res_slot, sh_res_cnt, sh_res_base, sh_started, &sh_pool,
-                    sh_warp_act, sh_warp_knd, &sh_share, &sh_tail, tail_groups};
+                    sh_warp_act, sh_warp_knd, &sh_share, &sh_tail, tail_groups, sh_act_count, sh_flags};
     for (int s = threadIdx.x; s < E.max_requests; s += blockDim.x) {
         sh_ok[s] = 0u;
         sh_held[s] = 0;
@@ -1174,6 +1177,8 @@ __global__ void __launch_bounds__(T == 1 ? 640 : 256, 1) engine_chunk_kernel(con
         sh_chunk = c == 0u || c > E.chunk_blocks ? E.chunk_blocks : c;
         sh_share = sh_chunk - sh_chunk / kPoolDiv;
     }
+    if (threadIdx.x < kNumKinds) sh_act_count[threadIdx.x] = E.act_count[threadIdx.x];
+    if (threadIdx.x < 2) sh_flags[threadIdx.x] = threadIdx.x == 0 ? *E.strict : *E.claim_warps;
     if (threadIdx.x < 32) {
         sh_res_slot[threadIdx.x] = -1;
         sh_res_cnt[threadIdx.x] = 0;
@@ -1185,10 +1190,10 @@ __global__ void __launch_bounds__(T == 1 ? 640 : 256, 1) engine_chunk_kernel(con
     __syncthreads();
     {
         int listed = 0;
-        for (int k = 0; k < kNumKinds; ++k) listed += E.act_count[k];
+        for (int k = 0; k < kNumKinds; ++k) listed += sh_act_count[k];
         for (int i = threadIdx.x; i < listed; i += blockDim.x) {
             int k = 0, j = i;
-            while (j >= E.act_count[k]) j -= E.act_count[k++];
+            while (j >= sh_act_count[k]) j -= sh_act_count[k++];
             const int s = E.act_list[k * E.max_requests + j];
             const SlotCtl &C = E.ctl[s];
             if (vload(C.state) != kSlotActive) continue;
@@ -1244,7 +1249,7 @@ __global__ void __launch_bounds__(T == 1 ? 640 : 256, 1) engine_chunk_kernel(con
     if (T == 1 && threadIdx.x < 32 && tail_groups > 0) {
         // dry from the start?  The queue heads as they are after this CTA's first claims.
         for (int k = 0; k < kNumKinds; ++k)
-            for (int j = lane; j < E.act_count[k]; j += 32) {
+            for (int j = lane; j < sh_act_count[k]; j += 32) {
                 const int s = E.act_list[k * E.max_requests + j];
                 if ((sh_ok[s] & 1u) && vload(E.ctl[s].head) >= E.slots[s].n_traj) atomicAnd(&sh_ok[s], ~1u);
             }
@@ -1407,11 +1412,11 @@ __global__ void __launch_bounds__(kSoloThreads, 1) solo_kernel(const __grid_cons
     __shared__ EngineDev E;
     __shared__ unsigned long long counters[kCntCount], res_base[32];
     __shared__ unsigned ok, share;
-    __shared__ int held, budget, pool, tail, claim, zeros[kNumKinds], counts[kNumKinds];
+    __shared__ int held, budget, pool, tail, flags[2], zeros[kNumKinds], counts[kNumKinds];
     __shared__ int res_slot[32], res_cnt[32], started[32], warp_act[32], warp_knd[32];
     unsigned *hist = reinterpret_cast<unsigned *>(tail_mem + tail_shared_bytes(kSoloThreads / 32));
     const CtaView V{&ok, &held, &budget, res_slot, res_cnt, res_base, started, &pool, warp_act, warp_knd, &share, &tail,
-                    tail_groups_of(1, kSoloThreads / 32)};
+                    tail_groups_of(1, kSoloThreads / 32), counts, flags};
     for (int b = threadIdx.x; b < a.nbins; b += blockDim.x) hist[b] = 0u;
     if (threadIdx.x < 32) {
         res_slot[threadIdx.x] = -1;
@@ -1437,10 +1442,7 @@ __global__ void __launch_bounds__(kSoloThreads, 1) solo_kernel(const __grid_cons
         E = EngineDev{};
         E.slots = &slot;
         E.ctl = &ctl;
-        E.strict = zeros;
-        E.claim_warps = &claim;
         E.act_list = zeros;
-        E.act_count = counts;
         E.counters = counters;
         E.max_requests = 1;
         E.n_lanes = gridDim.x * blockDim.x;
@@ -1448,7 +1450,8 @@ __global__ void __launch_bounds__(kSoloThreads, 1) solo_kernel(const __grid_cons
         held = budget = pool = tail = 0;
         share = 0x80000000u;   // blocks before the warps meet in any case (they go on)
         const unsigned long long warps = (end - first + 31) / 32;
-        claim = warps < kSoloThreads / 32 ? static_cast<int>(warps) : kSoloThreads / 32;
+        flags[0] = 0;
+        flags[1] = warps < kSoloThreads / 32 ? static_cast<int>(warps) : kSoloThreads / 32;
     }
     __syncthreads();
     Lane L[1];
@@ -1502,51 +1505,126 @@ __global__ void __launch_bounds__(kSoloThreads, 1) solo_kernel(const __grid_cons
         if (hist[b]) atomicAdd(&a.hist[b], static_cast<unsigned long long>(hist[b]));
 }
 
-// Fold completed id blocks, in id order, into each request's running sums; stop at the first
-// prefix meeting the relative-standard-error rule, or when every block is complete.
-__global__ void engine_scan_kernel(EngineDev E) {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
+// A prefix's exact sums: trajectories, escapes, out-of-range counts, sums of k and k^2.
+struct PrefixSums {
+    unsigned long long done, esc, under, over, s1_lo, s1_hi, s2_lo, s2_hi;
+    __device__ __forceinline__ void add(const PrefixSums &o) {
+        done += o.done;
+        esc += o.esc;
+        under += o.under;
+        over += o.over;
+        s1_lo += o.s1_lo;
+        s1_hi += o.s1_hi + (s1_lo < o.s1_lo ? 1ull : 0ull);
+        s2_lo += o.s2_lo;
+        s2_hi += o.s2_hi + (s2_lo < o.s2_lo ? 1ull : 0ull);
+    }
+    __device__ __forceinline__ PrefixSums from(int lane) const {
+        PrefixSums r;
+        r.done = __shfl_sync(kFull, done, lane);
+        r.esc = __shfl_sync(kFull, esc, lane);
+        r.under = __shfl_sync(kFull, under, lane);
+        r.over = __shfl_sync(kFull, over, lane);
+        r.s1_lo = __shfl_sync(kFull, s1_lo, lane);
+        r.s1_hi = __shfl_sync(kFull, s1_hi, lane);
+        r.s2_lo = __shfl_sync(kFull, s2_lo, lane);
+        r.s2_hi = __shfl_sync(kFull, s2_hi, lane);
+        return r;
+    }
+};
+
+// The relative-standard-error rule on a prefix (IEEE double, each operation rounded).
+__device__ __forceinline__ bool stop_rule(const SlotDev *S, const PrefixSums &P) {
+    if (P.esc < 2) return false;
+    const double n = static_cast<double>(P.esc);
+    const double s1 = u128_to_d(P.s1_lo, P.s1_hi);
+    const double s2 = u128_to_d(P.s2_lo, P.s2_hi);
+    const double mk = __ddiv_rn(s1, n);
+    double vk = __ddiv_rn(__dsub_rn(s2, __dmul_rn(s1, mk)), __dsub_rn(n, 1.0));
+    if (vk < 0.0) vk = 0.0;
+    const double mx = S->output == FPT_OUT_TIME ? __dmul_rn(S->out_b, mk)
+                                                : __dadd_rn(S->out_a, __dmul_rn(S->out_b, mk));
+    const double se = __dmul_rn(fabs(S->out_b), __dsqrt_rn(__ddiv_rn(vk, n)));
+    return se <= __dmul_rn(S->stop_rse, fabs(mx));
+}
+
+// After a launch, one warp per request: folds its completed id blocks, in id order and 32 at a time
+// (each lane one block, sums to its block by a scan over the lanes, the stop rule on each prefix),
+// into its running sums; it is finished at the first prefix that meets the rule, or when every
+// block is complete.  Then the status of every slot in use and the counters go straight to the
+// host's pinned memory, where two copies behind this kernel would each cost a step of the graph.
+__global__ void engine_scan_kernel(EngineDev E, SlotCtl *h_ctl, unsigned long long *h_counters) {
+    const int s = static_cast<int>((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+    if (blockIdx.x == 0 && threadIdx.x < kCntCount) h_counters[threadIdx.x] = E.counters[threadIdx.x];
     if (s >= E.max_requests) return;
     SlotCtl *C = E.ctl + s;
-    if (C->state != kSlotActive) return;
-    const SlotDev *S = E.slots + s;
-    // entries suspended during the launch become available to the next launch's refills
-    C->park_avail += static_cast<int>(C->park_tail - C->park_commit);
-    C->park_commit = C->park_tail;
-    unsigned p = C->prefix;
-    bool finished = false;
-    while (p < S->n_idblocks) {
-        const unsigned long long first = static_cast<unsigned long long>(p) * S->stop_block;
-        const unsigned long long left = S->n_traj - first;
-        const unsigned need = left < S->stop_block ? static_cast<unsigned>(left) : S->stop_block;
-        const IdBlockAcc &A = S->acc[p];
-        if (A.done < need) break;
-        C->n_done += A.done;
-        C->n_esc += A.escaped;
-        C->under += A.under;
-        C->over += A.over;
-        add_limbs(C->s1_lo, C->s1_hi, A.s1[0], A.s1[1], 0ull);
-        add_limbs(C->s2_lo, C->s2_hi, A.s2[0], A.s2[1], A.s2[2]);
-        ++p;
-        if (S->stop_rse > 0.0 && C->n_esc >= 2) {
-            const double n = static_cast<double>(C->n_esc);
-            const double s1 = u128_to_d(C->s1_lo, C->s1_hi);
-            const double s2 = u128_to_d(C->s2_lo, C->s2_hi);
-            const double mk = __ddiv_rn(s1, n);
-            double vk = __ddiv_rn(__dsub_rn(s2, __dmul_rn(s1, mk)), __dsub_rn(n, 1.0));
-            if (vk < 0.0) vk = 0.0;
-            const double mx = S->output == FPT_OUT_TIME ? __dmul_rn(S->out_b, mk)
-                                                        : __dadd_rn(S->out_a, __dmul_rn(S->out_b, mk));
-            const double se = __dmul_rn(fabs(S->out_b), __dsqrt_rn(__ddiv_rn(vk, n)));
-            if (se <= __dmul_rn(S->stop_rse, fabs(mx))) {
+    const int state = C->state;
+    if (state == kSlotFree) return;
+    if (state == kSlotActive) {
+        const SlotDev *S = E.slots + s;
+        unsigned p = C->prefix;
+        PrefixSums total{C->n_done, C->n_esc, C->under, C->over, C->s1_lo, C->s1_hi, C->s2_lo, C->s2_hi};
+        bool finished = false;
+        while (p < S->n_idblocks) {
+            const unsigned ib = p + static_cast<unsigned>(lane);
+            PrefixSums mine{};
+            bool complete = false;
+            if (ib < S->n_idblocks && ib >= p) {
+                const unsigned long long left = S->n_traj - static_cast<unsigned long long>(ib) * S->stop_block;
+                const unsigned need = left < S->stop_block ? static_cast<unsigned>(left) : S->stop_block;
+                const IdBlockAcc &A = S->acc[ib];
+                complete = A.done >= need;
+                if (complete) {
+                    mine.done = A.done;
+                    mine.esc = A.escaped;
+                    mine.under = A.under;
+                    mine.over = A.over;
+                    add_limbs(mine.s1_lo, mine.s1_hi, A.s1[0], A.s1[1], 0ull);
+                    add_limbs(mine.s2_lo, mine.s2_hi, A.s2[0], A.s2[1], A.s2[2]);
+                }
+            }
+            const unsigned gap = ~__ballot_sync(kFull, complete);
+            const int run = gap ? __ffs(gap) - 1 : 32;   // complete blocks from p on
+            if (run == 0) break;
+            if (lane >= run) mine = PrefixSums{};
+            if (lane == 0) mine.add(total);
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const PrefixSums o = mine.from((lane - off) & 31);
+                if (lane >= off) mine.add(o);
+            }
+            const bool stop = S->stop_rse > 0.0 && lane < run && stop_rule(S, mine);
+            const unsigned stops = __ballot_sync(kFull, stop);
+            const int last = stops ? __ffs(stops) - 1 : run - 1;
+            total = mine.from(last);
+            p += static_cast<unsigned>(last + 1);
+            if (stops) {
                 finished = true;
                 break;
             }
+            if (run < 32) break;
         }
+        if (p >= S->n_idblocks) finished = true;
+        if (lane == 0) {
+            // entries suspended during the launch become available to the next launch's refills
+            C->park_avail += static_cast<int>(C->park_tail - C->park_commit);
+            C->park_commit = C->park_tail;
+            C->n_done = total.done;
+            C->n_esc = total.esc;
+            C->under = total.under;
+            C->over = total.over;
+            C->s1_lo = total.s1_lo;
+            C->s1_hi = total.s1_hi;
+            C->s2_lo = total.s2_lo;
+            C->s2_hi = total.s2_hi;
+            C->prefix = p;
+            if (finished) C->state = kSlotFinished;
+        }
+        __syncwarp();
     }
-    C->prefix = p;
-    if (p >= S->n_idblocks) finished = true;
-    if (finished) C->state = kSlotFinished;
+    static_assert(sizeof(SlotCtl) % 8 == 0, "copied as 8-byte words");
+    const unsigned long long *src = reinterpret_cast<const unsigned long long *>(C);
+    unsigned long long *dst = reinterpret_cast<unsigned long long *>(h_ctl + s);
+    if (lane < static_cast<int>(sizeof(SlotCtl) / 8)) dst[lane] = src[lane];
 }
 
 }  // namespace
@@ -1605,10 +1683,10 @@ cudaError_t launch_solo(const Decoded &d, uint64_t seed, uint64_t traj_offset, u
     return cudaGetLastError();
 }
 
-cudaError_t launch_engine_scan(const EngineDev &E, cudaStream_t s) {
+cudaError_t launch_engine_scan(const EngineDev &E, SlotCtl *h_ctl, unsigned long long *h_counters, cudaStream_t s) {
     const unsigned block = 128;
-    const unsigned grid = (static_cast<unsigned>(E.max_requests) + block - 1) / block;
-    engine_scan_kernel<<<grid, block, 0, s>>>(E);
+    const unsigned grid = (static_cast<unsigned>(E.max_requests) * 32 + block - 1) / block;
+    engine_scan_kernel<<<grid, block, 0, s>>>(E, h_ctl, h_counters);
     return cudaGetLastError();
 }
 
