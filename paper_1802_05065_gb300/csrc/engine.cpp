@@ -70,6 +70,8 @@ struct Request {
     int slot = -1;
     Phase phase = kPending;
     bool released = false;
+    int readers = 0;                  // calls copying from its device memory at this moment
+    void *mem = nullptr;              // one device buffer of `bytes` for all of:
     IdBlockAcc *acc = nullptr;
     unsigned *hist = nullptr;
     long long *per_traj = nullptr;
@@ -118,13 +120,33 @@ uint64_t hist_rows(const fpt_params &p, uint64_t n_traj, uint32_t B) {
     return (n_traj + kHistRowIds - 1) / kHistRowIds;
 }
 
-size_t request_bytes(const fpt_params &p, uint64_t n_traj, uint32_t B, unsigned lanes) {
+// A request's device buffer: id-block accumulators and histogram rows (zeroed together), the
+// per-trajectory steps, the ring of suspended trajectories.
+struct RequestLayout {
+    size_t hist, per_traj, park, bytes;   // offsets (the accumulators lie at 0) and size
+};
+RequestLayout request_layout(const fpt_params &p, uint64_t n_traj, uint32_t B, unsigned lanes) {
+    const auto up = [](size_t x) { return (x + 255) / 256 * 256; };
     const uint64_t nb = (n_traj + B - 1) / B;
-    size_t bytes = nb * sizeof(IdBlockAcc) + hist_rows(p, n_traj, B) * static_cast<size_t>(p.hist_bins) * 4;
-    bytes += static_cast<size_t>(park_capacity(n_traj, lanes)) * sizeof(ParkEntry);
-    if (p.keep_per_traj) bytes += n_traj * 8;
-    return bytes;
+    RequestLayout l;
+    l.hist = up(nb * sizeof(IdBlockAcc));
+    l.per_traj = up(l.hist + hist_rows(p, n_traj, B) * static_cast<size_t>(p.hist_bins) * 4);
+    l.park = up(l.per_traj + (p.keep_per_traj ? n_traj * 8 : 0));
+    l.bytes = l.park + static_cast<size_t>(park_capacity(n_traj, lanes)) * sizeof(ParkEntry);
+    return l;
 }
+
+size_t request_bytes(const fpt_params &p, uint64_t n_traj, uint32_t B, unsigned lanes) {
+    return request_layout(p, n_traj, B, lanes).bytes;
+}
+
+// Device buffers of finished requests that an engine keeps for the next ones: at most so many, of
+// so many bytes together (they count against the engine's memory budget and go first).
+constexpr size_t kSpareBuffers = 16, kSpareBytes = 64u << 20;
+struct Spare {
+    void *p;
+    size_t bytes;
+};
 
 }  // namespace
 
@@ -200,6 +222,8 @@ struct fpt_engine {
     std::vector<uint64_t> slot_req;
     uint64_t next_id = 1;
     uint64_t budget = 0, mem_used = 0;
+    std::deque<Spare> spare;          // oldest first
+    size_t spare_bytes = 0;
     uint64_t iterations = 0;
     bool broken = false;
     std::string error;
@@ -228,17 +252,59 @@ fpt_status fail(fpt_engine *e, fpt_status st, const std::string &m) {
         }                                                                                \
     } while (0)
 
+// A finished request's buffer goes to the engine's spares, the oldest of which make room; work
+// enqueued for the next owner follows every use of this one on the engine's stream (mu held).
+void drop_spare(fpt_engine *e, size_t i) {
+    cudaFree(e->spare[i].p);
+    e->spare_bytes -= e->spare[i].bytes;
+    e->spare.erase(e->spare.begin() + static_cast<std::ptrdiff_t>(i));
+}
+
 void free_request_buffers(Request &R, fpt_engine *e) {
-    if (R.acc) cudaFree(R.acc);
-    if (R.hist) cudaFree(R.hist);
-    if (R.per_traj) cudaFree(R.per_traj);
-    if (R.park) cudaFree(R.park);
+    if (R.mem && R.bytes <= kSpareBytes) {
+        while (!e->spare.empty() && (e->spare.size() >= kSpareBuffers || e->spare_bytes + R.bytes > kSpareBytes))
+            drop_spare(e, 0);
+        e->spare.push_back({R.mem, R.bytes});
+        e->spare_bytes += R.bytes;
+    } else if (R.mem) {
+        cudaFree(R.mem);
+    }
+    R.mem = nullptr;
     R.acc = nullptr;
     R.hist = nullptr;
     R.per_traj = nullptr;
     R.park = nullptr;
     e->mem_used -= R.bytes;
     R.bytes = 0;
+}
+
+// A buffer of at least `bytes`: the smallest spare that is not twice too large, else a new one
+// (an allocation and its release cost ~100 us of a small request's time).
+cudaError_t take_buffer(fpt_engine *e, size_t bytes, Request &R) {
+    size_t best = e->spare.size();
+    for (size_t i = 0; i < e->spare.size(); ++i)
+        if (e->spare[i].bytes >= bytes && e->spare[i].bytes <= 2 * bytes + (64u << 10) &&
+            e->mem_used + e->spare[i].bytes <= e->budget &&
+            (best == e->spare.size() || e->spare[i].bytes < e->spare[best].bytes))
+            best = i;
+    if (best < e->spare.size()) {
+        R.mem = e->spare[best].p;
+        R.bytes = e->spare[best].bytes;
+        e->spare_bytes -= R.bytes;
+        e->spare.erase(e->spare.begin() + static_cast<std::ptrdiff_t>(best));
+    } else {
+        while (!e->spare.empty() && e->mem_used + e->spare_bytes + bytes > e->budget) drop_spare(e, 0);
+        cudaError_t ce = cudaMalloc(&R.mem, bytes);
+        if (ce == cudaErrorMemoryAllocation && !e->spare.empty()) {
+            cudaGetLastError();
+            while (!e->spare.empty()) drop_spare(e, 0);
+            ce = cudaMalloc(&R.mem, bytes);
+        }
+        if (ce != cudaSuccess) return ce;
+        R.bytes = bytes;
+    }
+    e->mem_used += R.bytes;
+    return cudaSuccess;
 }
 
 // Admit queued requests (called with mu held, on the driving thread).
@@ -263,19 +329,19 @@ fpt_status admit(fpt_engine *e) {
             continue;
         }
         const uint64_t nb = R.n_idblocks;
-        CK(cudaMalloc(&R.acc, nb * sizeof(IdBlockAcc)));
+        const RequestLayout lay = request_layout(R.params, R.n_traj, R.stop_block, e->lanes);
         const size_t hist_bytes = hist_rows(R.params, R.n_traj, R.stop_block) * static_cast<size_t>(R.params.hist_bins) * 4;
-        CK(cudaMalloc(&R.hist, hist_bytes));
-        CK(cudaMemsetAsync(R.acc, 0, nb * sizeof(IdBlockAcc), e->stream));
-        CK(cudaMemsetAsync(R.hist, 0, hist_bytes, e->stream));
+        CK(take_buffer(e, lay.bytes, R));
+        char *mem = static_cast<char *>(R.mem);
+        R.acc = reinterpret_cast<IdBlockAcc *>(mem);
+        R.hist = reinterpret_cast<unsigned *>(mem + lay.hist);
+        R.park = reinterpret_cast<ParkEntry *>(mem + lay.park);
+        R.park_cap = park_capacity(R.n_traj, e->lanes);
+        CK(cudaMemsetAsync(R.mem, 0, lay.hist + hist_bytes, e->stream));
         if (R.params.keep_per_traj) {
-            CK(cudaMalloc(&R.per_traj, R.n_traj * 8));
+            R.per_traj = reinterpret_cast<long long *>(mem + lay.per_traj);
             CK(cudaMemsetAsync(R.per_traj, 0xFF, R.n_traj * 8, e->stream));
         }
-        R.park_cap = park_capacity(R.n_traj, e->lanes);
-        CK(cudaMalloc(&R.park, static_cast<size_t>(R.park_cap) * sizeof(ParkEntry)));
-        R.bytes = bytes;
-        e->mem_used += bytes;
         const Decoded &d = R.dec;
         SlotDev &S = e->h_slots[s];
         std::memset(&S, 0, sizeof(S));
@@ -503,11 +569,23 @@ void process_status(fpt_engine *e) {
             C.inflight == 0) {
             e->slot_req[s] = 0;
             R.slot = -1;
-            if (R.released) {
+            if (R.released && R.readers == 0) {
                 free_request_buffers(R, e);
                 e->reqs.erase(R.id);
             }
         }
+    }
+}
+
+// Ends a call's copy from request R's device memory (mu held): a release that came meanwhile waits
+// for it.
+void end_read(fpt_engine *e, uint64_t id) {
+    auto it = e->reqs.find(id);
+    if (it == e->reqs.end()) return;
+    Request &R = *it->second;
+    if (--R.readers == 0 && R.released && R.slot < 0) {
+        free_request_buffers(R, e);
+        e->reqs.erase(it);
     }
 }
 
@@ -630,6 +708,7 @@ void destroy_all(fpt_engine *e) {
     e->n_flight = 0;
     for (auto &kv : e->reqs) free_request_buffers(*kv.second, e);
     e->reqs.clear();
+    while (!e->spare.empty()) drop_spare(e, 0);
     for (IterIO &B : e->iters) {
         if (B.exec) cudaGraphExecDestroy(B.exec);
         if (B.graph) cudaGraphDestroy(B.graph);
@@ -909,6 +988,18 @@ extern "C" fpt_status fpt_wait(fpt_engine *e, uint64_t req_id, double timeout_s,
     }
 }
 
+// Copies a finished request's device memory to the host and ends the read that its caller began.
+static cudaError_t read_back(fpt_engine *e, uint64_t req_id, void *dst, const void *src, size_t bytes) {
+    cudaError_t ce = cudaSetDevice(e->device);
+    if (ce == cudaSuccess && bytes) {
+        ce = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, e->io);
+        if (ce == cudaSuccess) ce = cudaStreamSynchronize(e->io);
+    }
+    std::lock_guard<std::mutex> lk(e->mu);
+    end_read(e, req_id);
+    return ce;
+}
+
 extern "C" fpt_status fpt_histogram(fpt_engine *e, uint64_t req_id, uint64_t *counts, int nbins,
                                     uint64_t *under, uint64_t *over) {
     if (!e || !counts) return fail(e, FPT_EINVAL, "NULL argument");
@@ -924,15 +1015,13 @@ extern "C" fpt_status fpt_histogram(fpt_engine *e, uint64_t req_id, uint64_t *co
         prefix = R->params.stop_rse > 0.0 ? R->prefix
                                           : static_cast<unsigned>(hist_rows(R->params, R->n_traj, R->stop_block));
         hist = R->hist;
+        ++R->readers;
         if (under) *under = R->sums.under;
         if (over) *over = R->sums.over;
     }
     std::vector<unsigned> rows(static_cast<size_t>(prefix) * nbins);
-    CK(cudaSetDevice(e->device));
-    if (!rows.empty()) {
-        CK(cudaMemcpyAsync(rows.data(), hist, rows.size() * 4, cudaMemcpyDeviceToHost, e->io));
-        CK(cudaStreamSynchronize(e->io));
-    }
+    const cudaError_t ce = read_back(e, req_id, rows.data(), hist, rows.size() * 4);
+    CK(ce);
     std::fill(counts, counts + nbins, 0ull);
     for (unsigned p = 0; p < prefix; ++p)
         for (int b = 0; b < nbins; ++b) counts[b] += rows[static_cast<size_t>(p) * nbins + b];
@@ -962,6 +1051,7 @@ static fpt_status per_traj_impl(fpt_engine *e, uint64_t req_id, int64_t *steps, 
         if (n > R->n_traj) return fail(e, FPT_EINVAL, "n exceeds n_traj");
         src = R->per_traj;
         d = R->dec;
+        ++R->readers;
     }
     std::vector<int64_t> tmp;
     int64_t *dst = steps;
@@ -969,11 +1059,8 @@ static fpt_status per_traj_impl(fpt_engine *e, uint64_t req_id, int64_t *steps, 
         tmp.resize(n);
         dst = tmp.data();
     }
-    CK(cudaSetDevice(e->device));
-    if (n) {
-        CK(cudaMemcpyAsync(dst, src, n * 8, cudaMemcpyDeviceToHost, e->io));
-        CK(cudaStreamSynchronize(e->io));
-    }
+    const cudaError_t ce = read_back(e, req_id, dst, src, n * 8);
+    CK(ce);
     if (xs)
         for (uint64_t i = 0; i < n; ++i)
             xs[i] = dst[i] < 0 ? (d.output == FPT_OUT_TIME ? -1.0 : NAN)
@@ -1159,7 +1246,7 @@ extern "C" fpt_status fpt_release(fpt_engine *e, uint64_t req_id) {
         }
         return FPT_OK;
     }
-    if (R->slot < 0) {   // finished and its slot already recycled
+    if (R->slot < 0 && R->readers == 0) {   // finished and its slot already recycled
         free_request_buffers(*R, e);
         e->reqs.erase(req_id);
     }
