@@ -693,16 +693,20 @@ __device__ __forceinline__ int seek_work(Lane (&L)[T], const EngineDev &E, const
 // 26 ns per step mixed).  After each round of kRoundBlocks blocks or more the groups
 // are packed again if that makes them fewer.  The arithmetic of a trajectory is that of
 // run_blocks, bit for bit.  ns per step at 1 / 2 / 3 / 4 full warps per SM, the plain loop -> this:
-// overdamped Euler 31.5 / 31.5 / 31.5 / 31.5 -> 18.5 / 20.2 / 22.1 / 24.8, underdamped ramped Euler
-// 30.4 / 30.5 / 30.5 / 30.5 -> 14.8 / 18.8 / 22.8 / 27.5, underdamped Heun 40 -> 25 / 26 / 31 / 33;
-// a request of 1024 trajectories of 19 000 steps 3.7 -> 2.3 ms.
+// overdamped Euler 31.5 / 31.5 / 31.5 / 31.5 -> 17.5 / 18.5 / 21.2 / 22.8, underdamped ramped Euler
+// 30.4 / 30.5 / 30.5 / 30.5 -> 12.8 / 17.5 / 21.4 / 23.0, underdamped Heun 40 -> 24 / 25 / 29 / 33;
+// a request of 1024 trajectories of 19 000 steps 3.7 -> 2.2 ms.
 constexpr int kTailGroupsMax = 5;       // a quarter of the warps: one scheduler's
 constexpr int kTailMakers = 3;          // noise warps per group
 constexpr int kTailChunk = 3;           // blocks per chunk, one for each of them
 constexpr int kTailRing = 3 * kTailChunk;                     // blocks in a group's ring
 constexpr int kRoundBlocks = 256;
-constexpr int kNoiseFloats = 24;                              // per lane and block: 8 radii, 16 cos / sin
-constexpr int kNoiseBlock = 32 * kNoiseFloats;                // floats of one block of a group
+// Floats of one block of a group.  Euler: the 16 addends of the steps (noise and bias, formed by
+// the noise warps: an operation and half a load per step less in the chain's warp); Heun: 8 radii
+// and 16 cosines / sines, as its two stages take different biases.
+template <int H>
+constexpr int kNoiseBlock = 32 * (H == kEuler ? 16 : 24);
+constexpr int kNoiseBlockMax = 32 * 24;
 constexpr int kTailMinWarps = 8;
 
 // A request that runs without an engine (solo_kernel).
@@ -728,7 +732,7 @@ __host__ __device__ constexpr int tail_groups_of(int T, int warps) {
     return T != 1 || warps < kTailMinWarps ? 0 : (warps / 4 < kTailGroupsMax ? warps / 4 : kTailGroupsMax);
 }
 __host__ __device__ constexpr size_t tail_shared_bytes(int warps) {
-    return tail_groups_of(1, warps) == 0 ? 0 : static_cast<size_t>(tail_groups_of(1, warps)) * kTailRing * kNoiseBlock * 4 +
+    return tail_groups_of(1, warps) == 0 ? 0 : static_cast<size_t>(tail_groups_of(1, warps)) * kTailRing * kNoiseBlockMax * 4 +
                                                kTailGroupsMax * 32 * sizeof(TailLane);
 }
 
@@ -736,26 +740,34 @@ __device__ __forceinline__ void group_barrier(int group) {
     asm volatile("bar.sync %0, %1;" ::"r"(group + 1), "n"(32 * (1 + kTailMakers)) : "memory");
 }
 
-// One block of noise of one lane: tg[h] of call h at float4 (h, lane), its two radii at
-// float2 (h, lane) behind them.
-__device__ __forceinline__ void noise_store(float *block, int lane, int h, float2 rr, float4 tg) {
-    reinterpret_cast<float4 *>(block)[32 * h + lane] = tg;
-    reinterpret_cast<float2 *>(block + 16 * 32)[32 * h + lane] = rr;
-}
-__device__ __forceinline__ void noise_load(const float *block, int lane, int h, float2 &rr, float4 &tg) {
-    tg = reinterpret_cast<const float4 *>(block)[32 * h + lane];
-    rr = reinterpret_cast<const float2 *>(block + 16 * 32)[32 * h + lane];
-}
+// The noise of one call (steps 4 h .. 4 h + 3 of a block) of one lane, in shared memory as a float4
+// and, for Heun, a float2 behind the block's float4s.
+template <int H>
+struct TailCall {
+    float4 t;      // Euler: addends; Heun: cos, sin, cos, sin
+    float2 rr;     // Heun: the two radii
+    __device__ __forceinline__ void store(float *block, int lane, int h) const {
+        reinterpret_cast<float4 *>(block)[32 * h + lane] = t;
+        if constexpr (H == kHeun) reinterpret_cast<float2 *>(block + 16 * 32)[32 * h + lane] = rr;
+    }
+    __device__ __forceinline__ void load(const float *block, int lane, int h) {
+        t = reinterpret_cast<const float4 *>(block)[32 * h + lane];
+        if constexpr (H == kHeun) rr = reinterpret_cast<const float2 *>(block + 16 * 32)[32 * h + lane];
+    }
+};
 
-// Steps of call h of a block (4 h .. 4 h + 3).
+// Steps of call h of a block.
 template <int M, int H, int R, typename F>
-__device__ __forceinline__ void four_steps(Lane &L, int h, float2 rr, float4 tg, float gs, float gsl, F after) {
-    const float t[4] = {tg.x, tg.y, tg.z, tg.w};
+__device__ __forceinline__ void four_steps(Lane &L, int h, const TailCall<H> &n, float gs, float gsl, F after) {
+    const float t[4] = {n.t.x, n.t.y, n.t.z, n.t.w};
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
         const int s = 4 * h + q;
-        step_f32<M, H>(L.r, L.v, q < 2 ? rr.x : rr.y, t[q], bias_b0<H, R>(gs, gsl, s), bias_b1<H, R>(gs, gsl, s),
-                       L.dt, L.A, L.amp);
+        if constexpr (H == kEuler)
+            step_euler<M>(L.r, L.v, t[q], L.dt, L.A, __fmul_rn(-L.amp, L.dt));
+        else
+            step_f32<M, H>(L.r, L.v, q < 2 ? n.rr.x : n.rr.y, t[q], bias_b0<H, R>(gs, gsl, s),
+                           bias_b1<H, R>(gs, gsl, s), L.dt, L.A, L.amp);
         after(s);
     }
 }
@@ -765,7 +777,8 @@ static_assert(kTailGroupsMax <= kNumKinds, "the packing keeps the groups' kinds 
 extern __shared__ __align__(16) unsigned char tail_mem[];
 __device__ __forceinline__ TailLane *tail_lanes() { return reinterpret_cast<TailLane *>(tail_mem); }
 __device__ __forceinline__ float *tail_group_noise(int group) {
-    return reinterpret_cast<float *>(tail_mem + kTailGroupsMax * 32 * sizeof(TailLane)) + group * kTailRing * kNoiseBlock;
+    return reinterpret_cast<float *>(tail_mem + kTailGroupsMax * 32 * sizeof(TailLane)) +
+           group * kTailRing * kNoiseBlockMax;
 }
 struct TailShared {
     int count[kNumKinds];                   // lanes per kind (of the packing that is under way)
@@ -889,24 +902,23 @@ __device__ __forceinline__ void tail_integrate(const EngineDev &E, int group, in
     L.c_lo = 0u;
     if (T.slot >= 0) resume_from(L, E, T.slot, T);
     int n_active = L.slot >= 0 ? 1 : 0;
-    float gs, gsl;
+    float gs, gsl;   // Heun's bias line; an Euler step finds its bias in the noise
     bias_line(fmaf(L.nudt, L.Jf, L.gb), L.nudt, L.dt, gs, gsl);
-    const float *end = noise + kTailRing * kNoiseBlock, *cur = noise;   // this block's noise
-    float2 rr[kBlockPhilox];
-    float4 tg[kBlockPhilox];
+    const float *end = noise + kTailRing * kNoiseBlock<H>, *cur = noise;   // this block's noise
+    TailCall<H> calls[kBlockPhilox];
     group_barrier(group);
 #pragma unroll
-    for (int h = 0; h < kBlockPhilox; ++h) noise_load(cur, lane, h, rr[h], tg[h]);
+    for (int h = 0; h < kBlockPhilox; ++h) calls[h].load(cur, lane, h);
     int b = 0, b_count = 0, left = kTailChunk;   // blocks done, blocks counted, blocks left of the chunk
     for (int parity = 0;;) {
-        if constexpr (R) bias_line(fmaf(L.nudt, L.Jf, L.gb), L.nudt, L.dt, gs, gsl);
-        const float *next = cur + kNoiseBlock == end ? noise : cur + kNoiseBlock;
+        if constexpr (R && H == kHeun) bias_line(fmaf(L.nudt, L.Jf, L.gb), L.nudt, L.dt, gs, gsl);
+        const float *next = cur + kNoiseBlock<H> == end ? noise : cur + kNoiseBlock<H>;
         const float r0 = L.r, v0 = L.v;
         float mx = -INFINITY;
 #pragma unroll
         for (int h = 0; h < kBlockPhilox; ++h) {
-            four_steps<M, H, R>(L, h, rr[h], tg[h], gs, gsl, [&](int) { mx = fmaxf(mx, L.r); });
-            noise_load(next, lane, h, rr[h], tg[h]);
+            four_steps<M, H, R>(L, h, calls[h], gs, gsl, [&](int) { mx = fmaxf(mx, L.r); });
+            calls[h].load(next, lane, h);
         }
         L.c_lo += kBlockPhilox;
         if constexpr (R) L.Jf += static_cast<float>(kBlockSteps);
@@ -921,10 +933,9 @@ __device__ __forceinline__ void tail_integrate(const EngineDev &E, int group, in
                 L.v = v0;
 #pragma unroll
                 for (int h = 0; h < kBlockPhilox; ++h) {
-                    float2 rr2;
-                    float4 tg2;
-                    noise_load(cur, lane, h, rr2, tg2);
-                    four_steps<M, H, R>(L, h, rr2, tg2, gs, gsl, [&](int s) {
+                    TailCall<H> again;
+                    again.load(cur, lane, h);
+                    four_steps<M, H, R>(L, h, again, gs, gsl, [&](int s) {
                         if (L.r >= L.hb) phase_event(L, E, s);
                     });
                 }
@@ -947,7 +958,7 @@ __device__ __forceinline__ void tail_integrate(const EngineDev &E, int group, in
                 L.budget = 0xFFFFFFFFu;
             }
             over = !__any_sync(kFull, n_active > 0);
-            if constexpr (!R) bias_line(fmaf(L.nudt, L.Jf, L.gb), L.nudt, L.dt, gs, gsl);
+            if constexpr (!R && H == kHeun) bias_line(fmaf(L.nudt, L.Jf, L.gb), L.nudt, L.dt, gs, gsl);
         }
         cur = next;
         if (--left == 0 || b == round || over) {
@@ -974,18 +985,22 @@ __device__ __forceinline__ void tail_integrate(const EngineDev &E, int group, in
 }
 
 // One round of one of a group's noise warps: block `rank` of every chunk, two chunks ahead of the
-// integrating warp.
+// integrating warp.  Euler's addends take the bias line of set_progress and run_blocks: the base is
+// formed anew when the block count reaches a multiple of kRebaseBlocks.
+template <int H, int R>
 __device__ __forceinline__ void tail_noise(const EngineDev &E, int group, int rank, int round) {
     const int lane = threadIdx.x & 31;
     float *ring = tail_group_noise(group);
     const TailLane &T = tail_lanes()[32 * group + lane];
+    const SlotDev *S = E.slots + (T.slot >= 0 ? T.slot : 0);
     unsigned key0 = 0u, key1 = 0u, gid_lo = 0u, gid_hi = 0u, lo = 0u, hi = 0u;
-    float bmc = 0.0f;
+    float bmc = 0.0f, dt = 0.0f, nudt = 0.0f;
     if (T.slot >= 0) {
-        const SlotDev *S = E.slots + T.slot;
         key0 = S->key0;
         key1 = S->key1;
         bmc = S->bmc;
+        dt = S->dt;
+        nudt = S->nudt;
         gid_lo = T.gid_lo;
         gid_hi = T.gid_hi;
         const unsigned long long c = ((static_cast<unsigned long long>(T.c_hi) << 32) | T.c_lo) +
@@ -1001,26 +1016,42 @@ __device__ __forceinline__ void tail_noise(const EngineDev &E, int group, int ra
 #pragma unroll
     for (int r = 0; r < 7; ++r) asm volatile("" : "+r"(P.kb[r]));
     constexpr unsigned step = kBlockPhilox * kTailMakers;
-    const float *end = ring + kTailRing * kNoiseBlock;
-    float *block = ring + rank * kNoiseBlock;
+    float gb = 0.0f, Jf = 0.0f, gs = 0.0f, gsl = 0.0f;
+    const auto rebase = [&]() {   // bias base and steps since it at block count (hi : lo)
+        const unsigned long long c = (static_cast<unsigned long long>(hi) << 32) | lo, cb = c - c % kRebaseBlocks;
+        gb = static_cast<float>(S->gamma0 + S->nudt_d * static_cast<double>(4ull * cb));
+        Jf = static_cast<float>(4ull * (c - cb));
+        bias_line(fmaf(nudt, Jf, gb), nudt, dt, gs, gsl);
+    };
+    if constexpr (H == kEuler) rebase();
+    const float *end = ring + kTailRing * kNoiseBlock<H>;
+    float *block = ring + rank * kNoiseBlock<H>;
     int to_go = round - rank;                        // blocks from this one to the round's end
     for (int i = -2; kTailChunk * i < round; ++i) {   // makes chunk i + 2 while chunk i is used
         if (to_go > 0) {
+            if constexpr (H == kEuler && R) bias_line(fmaf(nudt, Jf, gb), nudt, dt, gs, gsl);
 #pragma unroll
             for (int h = 0; h < kBlockPhilox; ++h) {
                 const uint4 x = philox_lane_block(P, lo, static_cast<unsigned>(h));
-                float2 rr;
-                float4 tg;
-                bm_pair_f32(x.x, x.y, bmc, rr.x, tg.x, tg.y);
-                bm_pair_f32(x.z, x.w, bmc, rr.y, tg.z, tg.w);
-                noise_store(block, lane, h, rr, tg);
+                TailCall<H> n;
+                bm_pair_f32(x.x, x.y, bmc, n.rr.x, n.t.x, n.t.y);
+                bm_pair_f32(x.z, x.w, bmc, n.rr.y, n.t.z, n.t.w);
+                if constexpr (H == kEuler) {
+                    n.t.x = fmaf(n.rr.x, n.t.x, bias_b1<H, R>(gs, gsl, 4 * h));
+                    n.t.y = fmaf(n.rr.x, n.t.y, bias_b1<H, R>(gs, gsl, 4 * h + 1));
+                    n.t.z = fmaf(n.rr.y, n.t.z, bias_b1<H, R>(gs, gsl, 4 * h + 2));
+                    n.t.w = fmaf(n.rr.y, n.t.w, bias_b1<H, R>(gs, gsl, 4 * h + 3));
+                }
+                n.store(block, lane, h);
             }
         }
         to_go -= kTailMakers;
-        block += kTailChunk * kNoiseBlock;
-        if (block >= end) block -= kTailRing * kNoiseBlock;
+        block += kTailChunk * kNoiseBlock<H>;
+        if (block >= end) block -= kTailRing * kNoiseBlock<H>;
         lo += step;
-        if (__any_sync(kFull, lo < step)) {   // 2^32-block carry: new fixed words
+        Jf += static_cast<float>(4u * step);
+        // past a multiple of kRebaseBlocks: another bias base; past 2^32: new fixed words
+        if (__any_sync(kFull, (lo & (kRebaseBlocks - 1u)) < step)) {
             if (lo < step) {
                 ++hi;
                 PhiloxLane Q;
@@ -1030,12 +1061,14 @@ __device__ __forceinline__ void tail_noise(const EngineDev &E, int group, int ra
                 P.z1m = Q.z1m;
                 P.z2m = Q.z2m;
             }
+            if constexpr (H == kEuler) rebase();
         }
         if (i == -2) continue;   // the first barrier follows the second chunk
         group_barrier(group);
         if (i >= 0 && tail_sh.stop[i & 1][group]) break;
     }
 }
+static_assert((kRebaseBlocks & (kRebaseBlocks - 1u)) == 0u, "re-bases are found by a mask");
 static_assert(kTailChunk == kTailMakers, "a noise warp makes one block of each chunk");
 
 // Runs the CTA's trajectories, `groups` packed groups of them, at most `blocks` blocks of each, to
@@ -1080,7 +1113,10 @@ __device__ __noinline__ void tail_run(const EngineDev &E, int *held, int groups,
             default: tail_integrate<kOver, kHeun, kRamp>(E, group, round); break;
             }
         } else if (rank < kTailMakers) {
-            tail_noise(E, group, rank, round);
+            const int k = K >= 0 ? K : sh.kind[group];
+            if (k & 2) tail_noise<kHeun, kConstBias>(E, group, rank, round);
+            else if (k & 4) tail_noise<kEuler, kRamp>(E, group, rank, round);
+            else tail_noise<kEuler, kConstBias>(E, group, rank, round);
         }
         blocks -= static_cast<unsigned>(round);
         __syncthreads();

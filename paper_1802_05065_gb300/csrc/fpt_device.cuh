@@ -220,20 +220,24 @@ __device__ __forceinline__ float bias_b1(float base, float slope, int s) {
 // r is the phase wrapped to [-pi, pi); the caller restores the range and counts windings.
 // Every rounding is explicit (fmaf / __fmul_rn / __fadd_rn), so all kernels that take this step
 // agree bit for bit.
+// The Euler step from its addend q = fmaf(rr, trig, b1), which does not depend on the state.
+template <int M>
+__device__ __forceinline__ void step_euler(float &r, float &v, float q, float dt, float A, float c) {
+    const float s = __sinf(r);
+    if constexpr (M == kUnder) {
+        const float vn = fmaf(c, s, fmaf(A, v, q));
+        r = fmaf(dt, v, r);
+        v = vn;
+    } else {
+        r = fmaf(c, s, __fadd_rn(r, q));
+    }
+}
 template <int M, int H>
 __device__ __forceinline__ void step_f32(float &r, float &v, float rr, float trig, float b0,
                                          float b1, float dt, float A, float amp) {
     const float c = __fmul_rn(-amp, dt);
     if constexpr (H == kEuler) {
-        const float s = __sinf(r);
-        const float q = fmaf(rr, trig, b1);    // dt gamma_k + sigma z: independent of the state
-        if constexpr (M == kUnder) {
-            const float vn = fmaf(c, s, fmaf(A, v, q));
-            r = fmaf(dt, v, r);
-            v = vn;
-        } else {
-            r = fmaf(c, s, __fadd_rn(r, q));
-        }
+        step_euler<M>(r, v, fmaf(rr, trig, b1), dt, A, c);
     } else {
         const float hc = __fmul_rn(0.5f, c);
         const float q0 = fmaf(rr, trig, b0);
