@@ -516,9 +516,10 @@ __device__ __forceinline__ bool grant(const CtaView &V, unsigned &limit) {
 }
 
 // This warp's lanes after an event, for the CTA's view, and whether the CTA has run dry
-// (warp-collective): nothing left to claim or resume in any listed request, no reservoir, and few
-// enough trajectories left for its groups.  Then the warps are called together (V.tail); the
-// exact counts are taken when they have met.
+// (warp-collective): nothing left to claim or resume in any listed request, no reservoir, and so few
+// trajectories left that they fit its groups, or three quarters of the warps that hold them.  Then
+// the warps are called together (V.tail); the exact counts are taken when they have met.  (Twelve
+// full warps take 52 ns per step, twenty sparse ones 82.)
 template <int T>
 __device__ __forceinline__ void look_dry(Lane (&L)[T], const EngineDev &E, const CtaView &V, int kind) {
     if constexpr (T == 1) {
@@ -533,8 +534,9 @@ __device__ __forceinline__ void look_dry(Lane (&L)[T], const EngineDev &E, const
         const int a = lane < warps ? vload(V.warp_act[lane]) : 0;
         const int total = __reduce_add_sync(kFull, a);
         const int kinds = __popc(__reduce_or_sync(kFull, a > 0 ? 1u << (vload(V.warp_knd[lane]) & 31) : 0u));
-        // groups: ceil(lanes / 32) of one kind, at most (lanes + 31 kinds) / 32 of several
-        if (total == 0 || total + (kinds > 1 ? 31 * kinds : 0) > 32 * V.tail_groups) return;
+        // warps they need: ceil(lanes / 32) of one kind, at most (lanes + 31 kinds) / 32 of several
+        const int need = (total + 31 * kinds) >> 5, holding = __popc(__ballot_sync(kFull, a > 0));
+        if (total == 0 || (need > V.tail_groups && 4 * need > 3 * holding)) return;
         bool work = lane < warps && vload(V.res_cnt[lane]) > 0;
         for (int k = 0; k < kNumKinds; ++k)
             for (int j = lane; j < V.act_count[k]; j += 32)
@@ -545,7 +547,7 @@ __device__ __forceinline__ void look_dry(Lane (&L)[T], const EngineDev &E, const
 
 // Blocks this warp may run before it looks again whether the CTA's warps are called together (a
 // look per block costs 2 % of a full CTA's rate).
-constexpr unsigned kLookBlocks = 32;
+constexpr unsigned kLookBlocks = 8;
 
 // More blocks for this warp (warp-collective): its own share kLookBlocks at a time, then the
 // CTA's pool; false when there are none or the warps are called together.
@@ -782,7 +784,7 @@ __device__ __forceinline__ float *tail_group_noise(int group) {
 }
 struct TailShared {
     int count[kNumKinds];                   // lanes per kind (of the packing that is under way)
-    int kind[kTailGroupsMax];               // of each group
+    int kind[32];                           // of each group (a CTA has at most 32 warps)
     int alive[kTailGroupsMax];              // its lanes with a trajectory, after a round
     int stop[2][kTailGroupsMax];            // group done, by parity of the chunk
 };
@@ -810,13 +812,13 @@ __device__ __forceinline__ int tail_count(Lane (&L)[1], int (&count)[kNumKinds],
     return groups;
 }
 
-// Packs the CTA's trajectories for tail_run (CTA-collective): their groups, or -1 with nothing
-// changed when they are more than the CTA can run.
-__device__ __forceinline__ int tail_pack(Lane (&L)[1], const CtaView &V, int kind) {
+// Packs the CTA's trajectories into groups of 32 of one kind in shared memory (CTA-collective) and
+// returns how many there are.  No more than the CTA has warps: each warp's trajectories are of one
+// kind, so packing never takes more groups than the warps that held them.
+__device__ __forceinline__ int tail_pack(Lane (&L)[1], int kind) {
     const int lane = threadIdx.x & 31;
     int base, at;
     const int groups = tail_count(L, tail_sh.count, kind, base, at);
-    if (groups > V.tail_groups) return -1;
     TailLane *lanes = tail_lanes();
     for (int i = threadIdx.x; i < 32 * groups; i += blockDim.x) lanes[i].slot = -1;
     __syncthreads();
@@ -838,6 +840,31 @@ __device__ __forceinline__ int tail_pack(Lane (&L)[1], const CtaView &V, int kin
             for (int n = tail_sh.count[k]; n > 0; n -= 32) tail_sh.kind[g++] = k;
     __syncthreads();
     return groups;
+}
+
+// More groups than tail_run takes: they go on in as many full warps (CTA-collective).
+__device__ __forceinline__ void tail_spread(Lane (&L)[1], const EngineDev &E, const CtaView &V, int groups, int &kind,
+                                            int &n_active) {
+    const int warp = static_cast<int>(threadIdx.x >> 5), lane = threadIdx.x & 31;
+    set_idle(L[0]);
+    n_active = 0;
+    kind = -1;
+    int act = 0;
+    if (warp < groups) {
+        kind = tail_sh.kind[warp];
+        const TailLane T = tail_lanes()[32 * warp + lane];
+        if (T.slot >= 0) {
+            resume_from(L[0], E, T.slot, T);
+            n_active = 1;
+        }
+        act = __popc(__ballot_sync(kFull, n_active > 0));
+    }
+    if (lane == 0) {
+        V.warp_act[warp] = act;
+        V.warp_knd[warp] = kind < 0 ? 0 : kind;
+    }
+    if (threadIdx.x == 0) *V.tail = 0;
+    __syncthreads();
 }
 
 // Lane state between launches.
@@ -1293,7 +1320,7 @@ __global__ void __launch_bounds__(T == 1 ? 640 : 256, 1) engine_chunk_kernel(con
         look_dry(L, E, V, kind < 0 ? 0 : kind);
     }
     unsigned limit = 0;
-    for (bool again = true; again;) {   // again: the call to the last trajectories came too early
+    for (bool again = true; again;) {   // again: the warps have met and go on with fewer of them
         again = false;
         while (b < limit || more(V, limit)) {
             if (kind < 0) {
@@ -1326,17 +1353,15 @@ __global__ void __launch_bounds__(T == 1 ? 640 : 256, 1) engine_chunk_kernel(con
                 if (lane == 0 && kind >= 0) atomicMax(&sh_done, static_cast<int>(b));
                 __syncthreads();
                 if (sh_tail != 0) {
-                    const int groups = tail_pack(L, V, kind);
-                    if (groups >= 0) {
+                    const int groups = tail_pack(L, kind);
+                    if (groups <= tail_groups) {
                         if (lane == 0) E.warp_cursor[warp] = cursor;
                         add_counters(E, useful, n_esc, n_cens);
                         const unsigned done = static_cast<unsigned>(sh_done);
                         tail_run<-1>(E, sh_held, groups, sh_chunk > done ? sh_chunk - done : 0u);
                         return;
                     }
-                    __syncthreads();   // a warp found more work after the call: go on as before
-                    if (threadIdx.x == 0) sh_tail = 0;
-                    __syncthreads();
+                    tail_spread(L, E, V, groups, kind, n_active);
                     again = true;
                 }
             }
@@ -1512,13 +1537,14 @@ __global__ void __launch_bounds__(kSoloThreads, 1) solo_kernel(const __grid_cons
             run_blocks<M, H, R, 1>(L, E, V, b, n_active, cursor, useful, n_esc, n_cens, limit);
         __syncthreads();
         if (tail != 0) {
-            const int groups = tail_pack(L, V, kind);
-            if (groups >= 0) {
+            const int groups = tail_pack(L, kind);
+            if (groups <= V.tail_groups) {
                 tail_run<kind>(E, &held, groups, ~0ull);
                 break;
             }
-            __syncthreads();
-            if (threadIdx.x == 0) tail = 0;
+            int k = kind;
+            tail_spread(L, E, V, groups, k, n_active);
+            continue;
         }
         if (!__syncthreads_or(n_active > 0)) break;
     }

@@ -64,3 +64,11 @@ def test_kinds_mixed():
     reqs = [(d, 700 + 301 * i, 50 + i) for i, d in enumerate(KINDS)]
     for k, (d, n, s) in zip(_run(reqs, chunk_steps=4096), reqs):
         assert (k == _plain(d, n, s)).all()
+
+
+@pytest.mark.parametrize("threads", [256, 640])
+def test_full_ctas_thin_out(threads):
+    """More trajectories than lanes, of two kinds: warps meet several times and go on with fewer."""
+    reqs = [(OVER, 97280 + 77, 60), (UNDER, 60001, 61)]
+    for k, (d, n, s) in zip(_run(reqs, chunk_steps=4096, threads_per_block=threads), reqs):
+        assert (k == _plain(d, n, s)).all()
