@@ -67,6 +67,7 @@ struct Request {
     fpt_params params{};
     Decoded dec;
     uint64_t n_traj = 0, seed = 0;
+    uint64_t claim_end0 = 0;          // ids handed out from the first launch on (claim_end)
     int slot = -1;
     Phase phase = kPending;
     bool released = false;
@@ -388,7 +389,10 @@ fpt_status admit(fpt_engine *e) {
             CK(cudaStreamSynchronize(e->stream));   // the payload is host memory we free below
             R.restore.clear();
             R.restore.shrink_to_fit();
+        } else if (R.params.stop_rse > 0.0) {
+            C.claim_blocks = claim_blocks_for(1.0 / (R.params.stop_rse * R.params.stop_rse), R.stop_block, 0);
         }
+        R.claim_end0 = claim_end(R.n_traj, R.stop_block, C.claim_blocks);
         C.state = kSlotActive;
         CK(cudaMemcpyAsync(e->d_ctl + s, &C, sizeof(SlotCtl), cudaMemcpyHostToDevice, e->stream));
         e->slot_req[s] = R.id;
@@ -409,6 +413,12 @@ fpt_status admit(fpt_engine *e) {
 // Whether the last processed status describes request R (and not its slot's previous occupant).
 bool fresh(const fpt_engine *e, const Request &R) {
     return e->status_seq != UINT64_MAX && e->status_seq >= R.admit_seq;
+}
+
+// Ids of R still to be handed out, from its status.
+uint64_t unclaimed(const Request &R, const SlotCtl &C) {
+    const uint64_t end = claim_end(R.n_traj, R.stop_block, C.claim_blocks);
+    return C.head < end ? end - C.head : 0;
 }
 
 void build_lists(fpt_engine *e, IterIO &B) {
@@ -444,11 +454,10 @@ void build_lists(fpt_engine *e, IterIO &B) {
             if (R.phase != kRunning || R.suspending) continue;
             const SlotCtl &C = e->h_ctl[s];
             if (fresh(e, R) && C.state == kSlotActive) {
-                const uint64_t head = std::min<uint64_t>(C.head, R.n_traj);
-                work += static_cast<int64_t>(R.n_traj - head) + std::max(C.inflight, 0) +
+                work += static_cast<int64_t>(unclaimed(R, C)) + std::max(C.inflight, 0) +
                         std::max(C.park_avail, 0);
             } else {
-                work += static_cast<int64_t>(R.n_traj);   // admitted for the coming launch
+                work += static_cast<int64_t>(R.claim_end0);   // admitted for the coming launch
             }
         }
         const int64_t per_warp = 32ll * e->T * e->grid;
@@ -483,11 +492,10 @@ void build_lists(fpt_engine *e, IterIO &B) {
         // the end of that launch (waiting for its first status would cost two launches).
         const bool known = fresh(e, R);
         if (known && C.state != kSlotActive) continue;     // finishing
-        int64_t inflight = 0, remaining = static_cast<int64_t>(R.n_traj);
+        int64_t inflight = 0, remaining = static_cast<int64_t>(R.claim_end0);
         if (known) {
-            const int64_t unclaimed = C.head < R.n_traj ? static_cast<int64_t>(R.n_traj - C.head) : 0;
             inflight = C.inflight;
-            remaining = unclaimed + std::max(C.park_avail, 0);
+            remaining = static_cast<int64_t>(unclaimed(R, C)) + std::max(C.park_avail, 0);
         }
         const int64_t want = std::min<int64_t>(share, inflight + remaining);
         if (remaining > 0 && inflight < want / 2) deficit[R.dec.kind] += want - inflight;

@@ -129,7 +129,7 @@ struct SlotCtl {
     int inflight;              // lanes integrating a trajectory of this request
     int state;                 // kSlot*
     unsigned int prefix;       // id blocks folded into the running sums
-    unsigned int reserved;
+    unsigned int claim_blocks; // id blocks handed out so far (stop rule), 0: no limit; see claim_end
     unsigned long long n_done, n_esc, s1_lo, s1_hi, s2_lo, s2_hi, under, over;
     // suspended-trajectory ring: pushes at launch end, committed by the scan, popped by refill
     unsigned park_tail, park_head, park_commit;
@@ -137,6 +137,29 @@ struct SlotCtl {
     int park_used;             // entries pushed and not yet taken (bounds the ring)
     int reserved2;
 };
+
+// Ids of a request that are handed out: all of them, or with a stop rule as many id blocks as its
+// result is expected to take.  A request that stops after 12 288 of 262 144 trajectories otherwise
+// fills every lane with ids that are never used, at 82 ns per step instead of 22 (measured: the
+// mixed batch of 12 requests 34.9 -> 18.9 ms).  The expectation starts from a coefficient of
+// variation of 1 (an activated escape is close to exponential) and follows the prefix folded so
+// far; the scan raises it until the rule is met, so results do not depend on it.
+FPT_HD inline uint64_t claim_end(uint64_t n_traj, uint32_t stop_block, uint32_t claim_blocks) {
+    const uint64_t ids = static_cast<uint64_t>(claim_blocks) * stop_block;
+    return claim_blocks == 0 || ids > n_traj ? n_traj : ids;
+}
+
+// Blocks to hand out when `prefix` of them are folded and the rule needs `ids` trajectories in all:
+// a quarter more than that, half as much again as is folded, and never fewer ids ahead than two
+// warps per SM, which run no slower than one.
+FPT_HD inline uint32_t claim_blocks_for(double ids, uint32_t stop_block, uint32_t prefix) {
+    const double B = stop_block, p = prefix, ahead = 64.0 * 152.0;
+    double blocks = 1.25 * ids / B;
+    if (!(blocks < 4.0e9)) return 0;   // also a NaN: no limit
+    if (blocks < 1.5 * p) blocks = 1.5 * p;
+    if (blocks < p + ahead / B) blocks = p + ahead / B;
+    return blocks + 2.0 < 4.0e9 ? static_cast<uint32_t>(blocks + 2.0) : 0u;
+}
 
 struct LaneSoA {
     float *r, *v, *hb;

@@ -423,6 +423,11 @@ __device__ __forceinline__ int refill(Lane (&L)[T], const EngineDev &E, const Ct
                 //    Only warps that start a trajectory at least every 8 blocks keep one: for
                 //    long trajectories the ids would mostly return to the ring unused.
                 if (want > got && (V.ok[s] & 1u)) {
+                    const unsigned long long end = claim_end(n_traj, E.slots[s].stop_block, C->claim_blocks);
+                    // a limited request: look before claiming (warps that look at once go past it)
+                    if (end < n_traj && vload(C->head) >= end) atomicAnd(&V.ok[s], ~1u);
+                }
+                if (want > got && (V.ok[s] & 1u)) {
                     const int wn = want - got;
                     int extra = 0;
                     if (V.res_cnt[wl] == 0 && !capped && b > 0 && 8u * static_cast<unsigned>(V.started[wl]) >= b) {
@@ -451,7 +456,8 @@ __device__ __forceinline__ int refill(Lane (&L)[T], const EngineDev &E, const Ct
                         }
                     }
                     if (extra > keep) atomicAdd(&V.budget[s], extra - keep);
-                    if (base + static_cast<unsigned long long>(cl) >= n_traj) atomicAnd(&V.ok[s], ~1u);
+                    if (base + static_cast<unsigned long long>(cl) >= claim_end(n_traj, E.slots[s].stop_block, C->claim_blocks))
+                        atomicAnd(&V.ok[s], ~1u);
                 }
                 if (got) {
                     atomicAdd(&C->inflight, got);
@@ -1260,7 +1266,8 @@ __global__ void __launch_bounds__(T == 1 ? 640 : 256, 1) engine_chunk_kernel(con
             const int s = E.act_list[k * E.max_requests + j];
             const SlotCtl &C = E.ctl[s];
             if (vload(C.state) != kSlotActive) continue;
-            sh_ok[s] = (vload(C.head) < E.slots[s].n_traj ? 1u : 0u) | (vload(C.park_avail) > 0 ? 2u : 0u);
+            sh_ok[s] = (vload(C.head) < claim_end(E.slots[s].n_traj, E.slots[s].stop_block, C.claim_blocks) ? 1u : 0u) |
+                       (vload(C.park_avail) > 0 ? 2u : 0u);
             // reservoir room: what the ring can still take beyond one entry per lane (the most
             // suspensions of this launch could add), shared equally by the CTAs
             const long long room = static_cast<long long>(E.slots[s].park_cap) - vload(C.park_used) -
@@ -1314,7 +1321,9 @@ __global__ void __launch_bounds__(T == 1 ? 640 : 256, 1) engine_chunk_kernel(con
         for (int k = 0; k < kNumKinds; ++k)
             for (int j = lane; j < sh_act_count[k]; j += 32) {
                 const int s = E.act_list[k * E.max_requests + j];
-                if ((sh_ok[s] & 1u) && vload(E.ctl[s].head) >= E.slots[s].n_traj) atomicAnd(&sh_ok[s], ~1u);
+                if ((sh_ok[s] & 1u) &&
+                    vload(E.ctl[s].head) >= claim_end(E.slots[s].n_traj, E.slots[s].stop_block, E.ctl[s].claim_blocks))
+                    atomicAnd(&sh_ok[s], ~1u);
             }
         __syncwarp();
         look_dry(L, E, V, kind < 0 ? 0 : kind);
@@ -1594,8 +1603,11 @@ struct PrefixSums {
     }
 };
 
-// The relative-standard-error rule on a prefix (IEEE double, each operation rounded).
-__device__ __forceinline__ bool stop_rule(const SlotDev *S, const PrefixSums &P) {
+// The relative-standard-error rule on a prefix (IEEE double, each operation rounded): whether the
+// standard error of the mean is at most stop_rse times the mean; `ids` gets the trajectories that
+// the rule is expected to need at this prefix's spread.
+__device__ __forceinline__ bool stop_rule(const SlotDev *S, const PrefixSums &P, double &ids) {
+    ids = 0.0;
     if (P.esc < 2) return false;
     const double n = static_cast<double>(P.esc);
     const double s1 = u128_to_d(P.s1_lo, P.s1_hi);
@@ -1606,7 +1618,10 @@ __device__ __forceinline__ bool stop_rule(const SlotDev *S, const PrefixSums &P)
     const double mx = S->output == FPT_OUT_TIME ? __dmul_rn(S->out_b, mk)
                                                 : __dadd_rn(S->out_a, __dmul_rn(S->out_b, mk));
     const double se = __dmul_rn(fabs(S->out_b), __dsqrt_rn(__ddiv_rn(vk, n)));
-    return se <= __dmul_rn(S->stop_rse, fabs(mx));
+    const double most = __dmul_rn(S->stop_rse, fabs(mx));
+    const double over = se / most;
+    ids = static_cast<double>(P.done) * over * over;
+    return se <= most;
 }
 
 // After a launch, one warp per request: folds its completed id blocks, in id order and 32 at a time
@@ -1623,9 +1638,11 @@ __global__ void engine_scan_kernel(EngineDev E, SlotCtl *h_ctl, unsigned long lo
     if (state == kSlotFree) return;
     if (state == kSlotActive) {
         const SlotDev *S = E.slots + s;
-        unsigned p = C->prefix;
+        const unsigned first = C->prefix;
+        unsigned p = first;
         PrefixSums total{C->n_done, C->n_esc, C->under, C->over, C->s1_lo, C->s1_hi, C->s2_lo, C->s2_hi};
         bool finished = false;
+        double need = 0.0;   // trajectories the stop rule is expected to take
         while (p < S->n_idblocks) {
             const unsigned ib = p + static_cast<unsigned>(lane);
             PrefixSums mine{};
@@ -1654,10 +1671,12 @@ __global__ void engine_scan_kernel(EngineDev E, SlotCtl *h_ctl, unsigned long lo
                 const PrefixSums o = mine.from((lane - off) & 31);
                 if (lane >= off) mine.add(o);
             }
-            const bool stop = S->stop_rse > 0.0 && lane < run && stop_rule(S, mine);
+            double ids = 0.0;
+            const bool stop = S->stop_rse > 0.0 && lane < run && stop_rule(S, mine, ids);
             const unsigned stops = __ballot_sync(kFull, stop);
             const int last = stops ? __ffs(stops) - 1 : run - 1;
             total = mine.from(last);
+            need = __shfl_sync(kFull, ids, last);
             p += static_cast<unsigned>(last + 1);
             if (stops) {
                 finished = true;
@@ -1680,6 +1699,10 @@ __global__ void engine_scan_kernel(EngineDev E, SlotCtl *h_ctl, unsigned long lo
             C->s2_hi = total.s2_hi;
             C->prefix = p;
             if (finished) C->state = kSlotFinished;
+            else if (C->claim_blocks != 0 && p > first) {
+                const unsigned claim = claim_blocks_for(need, S->stop_block, p);
+                if (claim == 0 || claim > C->claim_blocks) C->claim_blocks = claim;
+            }
         }
         __syncwarp();
     }

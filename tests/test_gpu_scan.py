@@ -61,3 +61,16 @@ def test_reused_buffers():
         for i, (n, bins, block) in enumerate([(3000, 50, 64), (3000, 50, 64), (2500, 300, 100), (40_000, 20, 4096),
                                               (900, 1000, 7), (3001, 50, 64), (39_000, 1, 4096), (5, 2, 1)] * 3):
             _check(eng, m, workloads.scaled(OVER, hist_bins=bins, stop_block=block), n, i)
+
+
+def test_stop_rule_hands_out_what_it_needs():
+    """A request that stops early does not fill the lanes with ids past its result (the first hand-out
+    is for 1.25 / rse^2 = 3125 or two warps per SM, 9728), and one whose rule is never met runs all."""
+    import paper_1802_05065_gb300 as m
+    for d, lo, hi in ((dict(stop_rse=0.02, stop_block=256), 1000, 25_000),
+                      (dict(stop_rse=1e-5, stop_block=256), 200_000, 200_000)):
+        with m.Engine(0, chunk_steps=1024) as eng:
+            p = workloads.scaled(OVER, max_steps=10**6, **d)
+            r = eng.wait(eng.submit(m.params_from(p), 200_000, 4), 120.0)
+            c = eng.counters()
+            assert lo <= r.n_used <= c["escapes"] + c["censored"] <= hi, (d, r.n_used, c)
