@@ -792,25 +792,23 @@ fpt_status create_impl(const fpt_engine_config *cfg_in, fpt_engine *e) {
     CK(cudaMalloc(&e->d_lists, list_ints(R) * sizeof(int)));
     CK(cudaMemsetAsync(e->d_lists, 0, list_ints(R) * sizeof(int), e->stream));
     const size_t L = e->lanes;
-    CK(cudaMalloc(&e->d_lane_mem, L * 4 * 10));
+    CK(cudaMalloc(&e->d_lane_mem, L * 4 * 8));
     const unsigned nwarps = static_cast<unsigned>(e->grid) * e->block / 32;
     CK(cudaMalloc(&e->d_warp_kind, nwarps * sizeof(int)));
     CK(cudaMalloc(&e->d_warp_cursor, nwarps * sizeof(unsigned)));
     CK(cudaMalloc(&e->d_counters, kCntCount * sizeof(unsigned long long)));
     CK(cudaMemsetAsync(e->d_ctl, 0, R * sizeof(SlotCtl), e->stream));
-    CK(cudaMemsetAsync(e->d_lane_mem, 0, L * 4 * 10, e->stream));
+    CK(cudaMemsetAsync(e->d_lane_mem, 0, L * 4 * 8, e->stream));
     char *m = static_cast<char *>(e->d_lane_mem);
     LaneSoA &ls = e->dev.lanes;
     ls.r = reinterpret_cast<float *>(m + 0 * L * 4);
     ls.v = reinterpret_cast<float *>(m + 1 * L * 4);
-    ls.hb = reinterpret_cast<float *>(m + 2 * L * 4);
-    ls.w = reinterpret_cast<int *>(m + 3 * L * 4);
-    ls.slot = reinterpret_cast<int *>(m + 4 * L * 4);
-    ls.c_lo = reinterpret_cast<unsigned *>(m + 5 * L * 4);
-    ls.c_hi = reinterpret_cast<unsigned *>(m + 6 * L * 4);
-    ls.gid_lo = reinterpret_cast<unsigned *>(m + 7 * L * 4);
-    ls.gid_hi = reinterpret_cast<unsigned *>(m + 8 * L * 4);
-    ls.budget = reinterpret_cast<unsigned *>(m + 9 * L * 4);
+    ls.w = reinterpret_cast<int *>(m + 2 * L * 4);
+    ls.slot = reinterpret_cast<int *>(m + 3 * L * 4);
+    ls.c_lo = reinterpret_cast<unsigned *>(m + 4 * L * 4);
+    ls.c_hi = reinterpret_cast<unsigned *>(m + 5 * L * 4);
+    ls.gid_lo = reinterpret_cast<unsigned *>(m + 6 * L * 4);
+    ls.gid_hi = reinterpret_cast<unsigned *>(m + 7 * L * 4);
     CK(cudaMemsetAsync(ls.slot, 0xFF, L * 4, e->stream));
     CK(cudaMemsetAsync(e->d_warp_kind, 0xFF, nwarps * sizeof(int), e->stream));
     {   // stagger the warps' round-robin cursors so the first claims spread over all requests

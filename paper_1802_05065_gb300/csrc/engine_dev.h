@@ -5,9 +5,9 @@
 //   SlotCtl[max_requests]     per-request work queue head, in-flight lane count, fair-share cap,
 //                             state and the running sums of the completed id-block prefix
 //   lane state, structure of arrays, one entry per lane (lanes = threads x T):
-//       r (wrapped phase), v, hb (upper event bound), w (winding), c (64-bit Philox block
+//       r (wrapped phase), v, w (winding), c (64-bit Philox block
 //       counter = Philox blocks of 4 steps consumed, a multiple of kBlockPhilox between kernel
-//       blocks), gid (64-bit trajectory id), slot, budget
+//       blocks), gid (64-bit trajectory id), slot
 //   per request: IdBlockAcc[n_idblocks] + u32 histogram rows [rows][hist_bins], rows = n_idblocks
 //       with a stop rule, ceil(n_traj / 2^31) without (+ optional int64 escape step per trajectory)
 #pragma once
@@ -162,9 +162,9 @@ FPT_HD inline uint32_t claim_blocks_for(double ids, uint32_t stop_block, uint32_
 }
 
 struct LaneSoA {
-    float *r, *v, *hb;
+    float *r, *v;
     int *w, *slot;
-    unsigned int *c_lo, *c_hi, *gid_lo, *gid_hi, *budget;
+    unsigned int *c_lo, *c_hi, *gid_lo, *gid_hi;
 };
 
 // Global counters; kCntCheck collects the violated bounds of a build with FPT_CHECK (bit per

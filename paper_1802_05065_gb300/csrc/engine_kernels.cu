@@ -521,11 +521,23 @@ __device__ __forceinline__ bool grant(const CtaView &V, unsigned &limit) {
     return g > 0;
 }
 
-// This warp's lanes after an event, for the CTA's view, and whether the CTA has run dry
-// (warp-collective): nothing left to claim or resume in any listed request, no reservoir, and so few
-// trajectories left that they fit its groups, or three quarters of the warps that hold them.  Then
-// the warps are called together (V.tail); the exact counts are taken when they have met.  (Twelve
+// Whether the trajectories the CTA's warps have published fit its groups, or three quarters of the
+// warps that hold them (warp-collective; the same for every warp between two publications).  (Twelve
 // full warps take 52 ns per step, twenty sparse ones 82.)
+__device__ __forceinline__ bool thinned_out(const CtaView &V) {
+    const int lane = threadIdx.x & 31, warps = static_cast<int>(blockDim.x >> 5);
+    const int a = lane < warps ? vload(V.warp_act[lane]) : 0;
+    const int total = __reduce_add_sync(kFull, a);
+    const int kinds = __popc(__reduce_or_sync(kFull, a > 0 ? 1u << (vload(V.warp_knd[lane]) & 31) : 0u));
+    // warps they need: ceil(lanes / 32) of one kind, at most (lanes + 31 kinds) / 32 of several
+    const int need = (total + 31 * kinds) >> 5, holding = __popc(__ballot_sync(kFull, a > 0));
+    return total > 0 && (need <= V.tail_groups || 4 * need <= 3 * holding);
+}
+
+// This warp's lanes after an event, for the CTA's view, and whether the CTA has run dry
+// (warp-collective): nothing left to claim or resume in any listed request, no reservoir, and
+// trajectories thinned out.  Then the warps are called together (V.tail); the exact counts are taken
+// when they have met.
 template <int T>
 __device__ __forceinline__ void look_dry(Lane (&L)[T], const EngineDev &E, const CtaView &V, int kind) {
     if constexpr (T == 1) {
@@ -537,12 +549,7 @@ __device__ __forceinline__ void look_dry(Lane (&L)[T], const EngineDev &E, const
             V.warp_knd[threadIdx.x >> 5] = kind;
         }
         __syncwarp();
-        const int a = lane < warps ? vload(V.warp_act[lane]) : 0;
-        const int total = __reduce_add_sync(kFull, a);
-        const int kinds = __popc(__reduce_or_sync(kFull, a > 0 ? 1u << (vload(V.warp_knd[lane]) & 31) : 0u));
-        // warps they need: ceil(lanes / 32) of one kind, at most (lanes + 31 kinds) / 32 of several
-        const int need = (total + 31 * kinds) >> 5, holding = __popc(__ballot_sync(kFull, a > 0));
-        if (total == 0 || (need > V.tail_groups && 4 * need > 3 * holding)) return;
+        if (!thinned_out(V)) return;
         bool work = lane < warps && vload(V.res_cnt[lane]) > 0;
         for (int k = 0; k < kNumKinds; ++k)
             for (int j = lane; j < V.act_count[k]; j += 32)
@@ -874,13 +881,13 @@ __device__ __forceinline__ void tail_spread(Lane (&L)[1], const EngineDev &E, co
 }
 
 // Lane state between launches.
-__device__ __forceinline__ void store_lane(const EngineDev &E, unsigned i, const Lane &L) {
+template <typename State>
+__device__ __forceinline__ void store_lane(const EngineDev &E, unsigned i, const State &L) {
     if (!checked(E, i < E.n_lanes, kChkLane)) return;
     E.lanes.slot[i] = L.slot;
     if (L.slot < 0) return;
     E.lanes.r[i] = L.r;
     E.lanes.v[i] = L.v;
-    E.lanes.hb[i] = L.hb;
     E.lanes.w[i] = L.w;
     E.lanes.c_lo[i] = L.c_lo;
     E.lanes.c_hi[i] = L.c_hi;
@@ -888,19 +895,15 @@ __device__ __forceinline__ void store_lane(const EngineDev &E, unsigned i, const
     E.lanes.gid_hi[i] = L.gid_hi;
 }
 __device__ __forceinline__ void load_lane(Lane &L, const EngineDev &E, unsigned i, int s) {
-    const SlotDev *S = E.slots + s;
-    L.slot = s;
-    L.r = E.lanes.r[i];
-    L.v = E.lanes.v[i];
-    L.hb = E.lanes.hb[i];
-    L.w = E.lanes.w[i];
-    L.c_lo = E.lanes.c_lo[i];
-    L.c_hi = E.lanes.c_hi[i];
-    L.gid_lo = E.lanes.gid_lo[i];
-    L.gid_hi = E.lanes.gid_hi[i];
-    L.esc = -1;
-    load_consts(L, S);
-    set_progress(L, S);
+    TailLane T;
+    T.r = E.lanes.r[i];
+    T.v = E.lanes.v[i];
+    T.w = E.lanes.w[i];
+    T.c_lo = E.lanes.c_lo[i];
+    T.c_hi = E.lanes.c_hi[i];
+    T.gid_lo = E.lanes.gid_lo[i];
+    T.gid_hi = E.lanes.gid_hi[i];
+    resume_from(L, E, s, T);
 }
 
 // A warp's share of the launch's counters (warp-collective).
@@ -1203,13 +1206,10 @@ __device__ __noinline__ void tail_run(const EngineDev &E, int *held, int groups,
     }
     if (!E.lanes.slot) return;
     // back into the lane state: group g in warp g
-    Lane L;
-    set_idle(L);
-    if (warp < groups) {
-        const TailLane T = lanes[32 * warp + lane];
-        if (T.slot >= 0) resume_from(L, E, T.slot, T);
-    }
-    store_lane(E, gtid, L);
+    TailLane T{};
+    T.slot = -1;
+    if (warp < groups) T = lanes[32 * warp + lane];
+    store_lane(E, gtid, T);
     if (lane == 0) E.warp_kind[gtid >> 5] = warp < groups ? sh.kind[warp] : -1;
 }
 
@@ -1246,6 +1246,13 @@ __global__ void __launch_bounds__(T == 1 ? 640 : 256, 1) engine_chunk_kernel(con
         sh_chunk = c == 0u || c > E.chunk_blocks ? E.chunk_blocks : c;
         sh_share = sh_chunk - sh_chunk / kPoolDiv;
     }
+    // this thread's lanes and this warp's kind, asked for before they are needed
+    int lane_slot[T];
+#pragma unroll
+    for (int t = 0; t < T; ++t)
+        lane_slot[t] = checked(E, t * nthreads + gtid < E.n_lanes, kChkLane) ? E.lanes.slot[t * nthreads + gtid] : -1;
+    int kind = E.warp_kind[warp];
+    unsigned cursor = E.warp_cursor[warp];
     if (threadIdx.x < kNumKinds) sh_act_count[threadIdx.x] = E.act_count[threadIdx.x];
     if (threadIdx.x < 2) sh_flags[threadIdx.x] = threadIdx.x == 0 ? *E.strict : *E.claim_warps;
     if (threadIdx.x < 32) {
@@ -1257,13 +1264,16 @@ __global__ void __launch_bounds__(T == 1 ? 640 : 256, 1) engine_chunk_kernel(con
         sh_warp_knd[threadIdx.x] = 0;
     }
     __syncthreads();
+    int listed = 0;
+    for (int k = 0; k < kNumKinds; ++k) listed += sh_act_count[k];
+    const auto listed_slot = [&](int i) {
+        int k = 0;
+        while (i >= sh_act_count[k]) i -= sh_act_count[k++];
+        return E.act_list[k * E.max_requests + i];
+    };
     {
-        int listed = 0;
-        for (int k = 0; k < kNumKinds; ++k) listed += sh_act_count[k];
         for (int i = threadIdx.x; i < listed; i += blockDim.x) {
-            int k = 0, j = i;
-            while (j >= sh_act_count[k]) j -= sh_act_count[k++];
-            const int s = E.act_list[k * E.max_requests + j];
+            const int s = listed_slot(i);
             const SlotCtl &C = E.ctl[s];
             if (vload(C.state) != kSlotActive) continue;
             sh_ok[s] = (vload(C.head) < claim_end(E.slots[s].n_traj, E.slots[s].stop_block, C.claim_blocks) ? 1u : 0u) |
@@ -1280,7 +1290,7 @@ __global__ void __launch_bounds__(T == 1 ? 640 : 256, 1) engine_chunk_kernel(con
 #pragma unroll
     for (int t = 0; t < T; ++t) {
         const unsigned i = t * nthreads + gtid;
-        int s = checked(E, i < E.n_lanes, kChkLane) ? E.lanes.slot[i] : -1;
+        int s = lane_slot[t];
         if (s >= 0 && !checked(E, s < E.max_requests, kChkSlot)) s = -1;
         if (s >= 0 && vload(E.ctl[s].state) != kSlotActive) {   // request finished or cancelled
             atomicSub(&E.ctl[s].inflight, 1);
@@ -1295,10 +1305,8 @@ __global__ void __launch_bounds__(T == 1 ? 640 : 256, 1) engine_chunk_kernel(con
         ++n_active;
     }
     __syncthreads();
-    int kind = E.warp_kind[warp];
     if (kind >= 0 && !checked(E, kind < kNumKinds, kChkKind)) kind = -1;
     if (!__any_sync(kFull, n_active > 0)) kind = -1;
-    unsigned cursor = E.warp_cursor[warp];
     unsigned long long useful = 0;
     unsigned n_esc = 0, n_cens = 0;
     unsigned b = 0;
@@ -1315,23 +1323,29 @@ __global__ void __launch_bounds__(T == 1 ? 640 : 256, 1) engine_chunk_kernel(con
             sh_warp_knd[threadIdx.x >> 5] = kind < 0 ? 0 : kind;
         }
     }
-    __syncthreads();
-    if (T == 1 && threadIdx.x < 32 && tail_groups > 0) {
-        // dry from the start?  The queue heads as they are after this CTA's first claims.
-        for (int k = 0; k < kNumKinds; ++k)
-            for (int j = lane; j < sh_act_count[k]; j += 32) {
-                const int s = E.act_list[k * E.max_requests + j];
-                if ((sh_ok[s] & 1u) &&
-                    vload(E.ctl[s].head) >= claim_end(E.slots[s].n_traj, E.slots[s].stop_block, E.ctl[s].claim_blocks))
-                    atomicAnd(&sh_ok[s], ~1u);
-            }
-        __syncwarp();
-        look_dry(L, E, V, kind < 0 ? 0 : kind);
+    // Dry from the start?  The queue heads as they are after this CTA's first claims; all warps see
+    // the same, so they go straight to the meeting.
+    bool dry = false;
+    {
+        bool work = false;
+        for (int i = threadIdx.x; i < listed; i += blockDim.x) {
+            const int s = listed_slot(i);
+            unsigned ok = vload(sh_ok[s]);
+            if (T == 1 && (ok & 1u) &&
+                vload(E.ctl[s].head) >= claim_end(E.slots[s].n_traj, E.slots[s].stop_block, E.ctl[s].claim_blocks))
+                ok = atomicAnd(&sh_ok[s], ~1u) & ~1u;
+            work |= (ok & 3u) != 0u;
+        }
+        work = __syncthreads_or(work) != 0;
+        if (T == 1 && tail_groups > 0 && !work && thinned_out(V)) {
+            dry = true;
+            if (threadIdx.x == 0) sh_tail = 1;
+        }
     }
     unsigned limit = 0;
     for (bool again = true; again;) {   // again: the warps have met and go on with fewer of them
         again = false;
-        while (b < limit || more(V, limit)) {
+        while (!dry && (b < limit || more(V, limit))) {
             if (kind < 0) {
                 kind = seek_work(L, E, V, n_active, cursor, b);
                 if (kind < 0) break;
@@ -1371,6 +1385,7 @@ __global__ void __launch_bounds__(T == 1 ? 640 : 256, 1) engine_chunk_kernel(con
                         return;
                     }
                     tail_spread(L, E, V, groups, kind, n_active);
+                    dry = false;
                     again = true;
                 }
             }
