@@ -129,6 +129,7 @@ void slot_constants(const Decoded &d, uint64_t seed, uint64_t traj_offset, SlotD
     S.hist_lo = d.hist_lo;
     S.hist_hi = d.hist_hi;
     S.hist_inv_w = d.hist_inv_w;
+    S.map = bin_map(d);
 }
 
 BinMap bin_map(const Decoded &d) {

@@ -14,13 +14,7 @@
 
 #include <cstdint>
 
-#if !defined(FPT_HD)
-#if defined(__CUDACC__)
-#define FPT_HD __host__ __device__
-#else
-#define FPT_HD
-#endif
-#endif
+#include "bin_map.h"
 
 namespace fpt {
 
@@ -102,6 +96,7 @@ struct SlotDev {
     // observable and histogram: x = out_a + out_b k
     int32_t output, hist_bins;
     double out_a, out_b, hist_lo, hist_hi, hist_inv_w;
+    BinMap map;               // the same bins in integers
     // prefix stop rule
     double stop_rse;
     uint32_t stop_block, n_idblocks;

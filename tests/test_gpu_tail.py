@@ -72,3 +72,16 @@ def test_full_ctas_thin_out(threads):
     reqs = [(OVER, 97280 + 77, 60), (UNDER, 60001, 61)]
     for k, (d, n, s) in zip(_run(reqs, chunk_steps=4096, threads_per_block=threads), reqs):
         assert (k == _plain(d, n, s)).all()
+
+
+@pytest.mark.parametrize("kw", [dict(chunk_steps=4096), dict(chunk_steps=80), dict(chunk_steps=4096, traj_per_thread=2)],
+                         ids=["4096", "80", "two per thread"])
+@pytest.mark.parametrize("d", [
+    workloads.scaled(OVER, dt=0.05), workloads.scaled(OVER, dt=0.2, max_steps=150, integrator="heun"),
+    workloads.scaled(UNDER, D=1.0, dt=0.05, max_steps=333), workloads.scaled(OVER, D=5.0, dt=0.05)],
+    ids=["380 steps", "heun", "censored", "a few blocks"])
+def test_short_trajectories_wait_for_each_other(d, kw):
+    """Escapes of several blocks are published together; launches end while some wait."""
+    n = 150_001 if kw["chunk_steps"] > 100 else 9_001
+    [k] = _run([(d, n, 5)], **kw)
+    assert (k == _plain(d, n, 5)).all()
