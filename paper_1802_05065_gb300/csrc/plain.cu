@@ -44,9 +44,9 @@ __device__ __forceinline__ uint32_t hi32(uint64_t x) { return static_cast<uint32
 // sake of one slow lane and a CTA's last trajectories have a scheduler to themselves.
 // Measured, against one trajectory per thread in 128-thread CTAs with noise and update in one
 // chain: 4096 underdamped trajectories of <= 20 000 steps 56.4 -> 21.1 ms (2.8 -> 1.05 us per
-// step), 65 536 overdamped ones of 19 000 steps on average 763 -> 226 ms (1.6 -> 5.5 Gstep/s).
+// step; 17.5 ms with F64Pair), 65 536 overdamped ones of 19 000 steps on average 763 -> 226 ms (1.6 -> 5.5 Gstep/s).
 constexpr int kF64Warps = 8;
-constexpr int kF64Blocks = 16;                  // Philox blocks per round
+constexpr int kF64Blocks = 16;                  // Philox blocks per round (fewer for a smaller step budget)
 constexpr int kF64Steps = 4 * kF64Blocks;       // steps per round
 constexpr int kF64Groups = 4;                   // groups of 32 lanes, one per scheduler
 
@@ -75,6 +75,83 @@ size_t f64_shared_bytes(int cols) {
     return static_cast<size_t>(cols) * (2 * kF64Steps * 8 + 3 * 8 + 3 * 4);
 }
 
+// The underdamped chain has room for a second warp: phi_{k+1} = phi_k + v_k dt does not wait for
+// sin phi_k, so one warp's sine of the new phase runs beside another's new velocity (Euler: 24
+// operations per step instead of 30), and Heun's two sines, of phi and of phi + v dt, run beside
+// each other (40 instead of 64).  With at most two groups in the CTA, group g's second warp is warp
+// groups + g, on a scheduler of its own; the two meet at a named barrier once per step and
+// exchange values through shared memory by the parity of the step.  Lanes that are done go on to the
+// round's end without effect.  4096 trajectories of <= 20 000 steps: 21.0 -> 17.5 ms.
+struct F64Pair {
+    double x[2][32], y[2][32];   // by parity: Euler sin phi and v; Heun's first warp q and a0 ...
+    double p[2][32];             // ... and its second sin p
+};
+__device__ __forceinline__ void pair_barrier(int group) {
+    asm volatile("bar.sync %0, 64;" ::"r"(group + 1) : "memory");
+}
+
+// One round of a group by its two warps (`second`: which of them); returns the step of the round at
+// whose end the phase reached th, or kF64Steps.  phi and v are the lane's at the start and the end;
+// Euler's first warp ends with phi, its second with v, Heun's with both.
+template <int H, int R, int A1>
+__device__ __forceinline__ int f64_pair_round(const PlainArgs &a, F64Pair &x, int group, bool second, const double *nz,
+                                              int cols, double &phi, double &v, double kd, double g_const,
+                                              long long th_key, int steps, int lim) {
+    const int lane = threadIdx.x & 31;
+    int hit = kF64Steps;
+    const auto sine = [&](double p) { return A1 ? sin(p) : __dmul_rn(a.amp, sin(p)); };
+    if constexpr (H == kEuler) {
+        if (second) x.y[0][lane] = v;
+        else x.x[0][lane] = sine(phi);
+        pair_barrier(group);
+    }
+    for (int t = 0; t < steps; ++t) {
+        double g = g_const, g0 = g_const;
+        if constexpr (R) {
+            if constexpr (H == kHeun) g0 = __dadd_rn(a.gamma0, __dmul_rn(a.nudt, kd));
+            if (H == kHeun || second) {
+                kd = __dadd_rn(kd, 1.0);
+                g = __dadd_rn(a.gamma0, __dmul_rn(a.nudt, kd));
+            }
+        }
+        const int now = t & 1, next = now ^ 1;
+        if constexpr (H == kEuler) {
+            if (second) {
+                const double acc = __dadd_rn(__dsub_rn(__dmul_rn(-a.alpha, v), x.x[now][lane]), g);
+                v = __dadd_rn(__dadd_rn(v, __dmul_rn(acc, a.dt)), nz[t * cols]);
+                x.y[next][lane] = v;
+            } else {
+                phi = __dadd_rn(phi, __dmul_rn(x.y[now][lane], a.dt));
+                if (hit == kF64Steps && t < lim && reached(phi, th_key)) hit = t;
+                x.x[next][lane] = sine(phi);
+            }
+            pair_barrier(group);
+        } else {
+            const double z = nz[t * cols];
+            double a0, q, sp;
+            if (second) {
+                sp = sine(__dadd_rn(phi, __dmul_rn(v, a.dt)));
+                x.p[now][lane] = sp;
+                pair_barrier(group);
+                q = x.x[now][lane];
+                a0 = x.y[now][lane];
+            } else {
+                a0 = __dadd_rn(__dsub_rn(__dmul_rn(-a.alpha, v), sine(phi)), g0);
+                q = __dadd_rn(__dadd_rn(v, __dmul_rn(a0, a.dt)), z);
+                x.x[now][lane] = q;
+                x.y[now][lane] = a0;
+                pair_barrier(group);
+                sp = x.p[now][lane];
+            }
+            const double a1 = __dadd_rn(__dsub_rn(__dmul_rn(-a.alpha, q), sp), g);
+            phi = __dadd_rn(phi, __dmul_rn(__dmul_rn(__dadd_rn(v, q), 0.5), a.dt));
+            v = __dadd_rn(__dadd_rn(v, __dmul_rn(__dmul_rn(__dadd_rn(a0, a1), 0.5), a.dt)), z);
+            if (hit == kF64Steps && t < lim && reached(phi, th_key)) hit = t;
+        }
+    }
+    return hit;
+}
+
 // R: ramped bias (0: gamma0 throughout, the value gamma0 + 0 k has); A1: the sin term's amplitude
 // is 1 (its product is exact and left out).
 template <int M, int H, int R, int A1>
@@ -82,6 +159,7 @@ __global__ void __launch_bounds__(32 * kF64Warps, 1) plain_f64_kernel(PlainArgs 
     extern __shared__ double f64_shared[];
     __shared__ unsigned long long sh_next, sh_end;   // the CTA's ids not yet started
     __shared__ int sh_cnt, sh_ticket;
+    __shared__ F64Pair pairs[M == kUnder ? 2 : 1];
     F64Lanes L;
     L.nz = f64_shared;
     L.phi = L.nz + 2 * kF64Steps * cols;
@@ -98,6 +176,8 @@ __global__ void __launch_bounds__(32 * kF64Warps, 1) plain_f64_kernel(PlainArgs 
         sh_cnt = 0;
     }
     const long long th_key = a.th == 0.0 ? -1ll : order_key(a.th);
+    const int blocks = a.max_steps < static_cast<uint64_t>(kF64Steps) ? static_cast<int>(a.max_steps + 3) / 4 : kF64Blocks;
+    const int steps = 4 * blocks;                    // of a round
     const double g_const = __dadd_rn(a.gamma0, __dmul_rn(a.nudt, 1.0));   // R = 0: nudt = 0
     __syncthreads();
     for (int buf = 0;; buf ^= 1) {
@@ -113,7 +193,7 @@ __global__ void __launch_bounds__(32 * kF64Warps, 1) plain_f64_kernel(PlainArgs 
                 if (live) {
                     phi = L.phi[p];
                     v = L.v[p];
-                    blk = L.blk[p] + (L.col[p] >= 0 ? kF64Blocks : 0);
+                    blk = L.blk[p] + (L.col[p] >= 0 ? blocks : 0);
                     idx = L.idx[p];
                 }
                 const unsigned m = __ballot_sync(0xFFFFFFFFu, live);
@@ -150,12 +230,39 @@ __global__ void __launch_bounds__(32 * kF64Warps, 1) plain_f64_kernel(PlainArgs 
         const int cnt = sh_cnt;
         if (cnt == 0) break;
         const int groups = (cnt + 31) >> 5;
+        const bool paired = M == kUnder && groups <= 2;
+        if (M == kUnder && paired && warp < 2 * groups) {
+            // both warps of a group take part in every step; lanes without noise yet idle
+            const int group = warp % groups, p = 32 * group + lane;
+            const bool second = warp >= groups, runs = p < cnt && L.col[p] >= 0;
+            double phi = runs ? L.phi[p] : 0.0, v = runs ? L.v[p] : 0.0;
+            const uint64_t k0 = runs ? 4ull * L.blk[p] : 0ull;
+            const uint64_t left = a.max_steps - k0;
+            const int lim = !runs ? 0 : left < static_cast<uint64_t>(steps) ? static_cast<int>(left) : steps;
+            const double *nz = L.nz + static_cast<size_t>(buf) * kF64Steps * cols + (runs ? L.col[p] : 0);
+            if (__any_sync(0xFFFFFFFFu, runs)) {   // the same for both warps
+                const int hit = f64_pair_round<H, R, A1>(a, pairs[group], group, second, nz, cols, phi, v,
+                                                         static_cast<double>(k0), g_const, th_key, steps, lim);
+                if (runs) {
+                    const bool esc = hit < kF64Steps;
+                    if (second) {
+                        L.v[p] = v;
+                    } else {
+                        L.phi[p] = phi;
+                        if (esc || k0 + static_cast<uint64_t>(lim) >= a.max_steps) {
+                            a.steps[first + L.idx[p]] = esc ? static_cast<int64_t>(k0 + static_cast<uint64_t>(hit) + 1ull) : -1;
+                            L.alive[p] = 0;
+                        }
+                    }
+                }
+            }
+        }
         const int p = 32 * warp + lane;
-        if (warp < groups && p < cnt && L.col[p] >= 0) {
+        if (!paired && warp < groups && p < cnt && L.col[p] >= 0) {
             double phi = L.phi[p], v = L.v[p];
             const uint64_t k0 = 4ull * L.blk[p];
             const uint64_t left = a.max_steps - k0;
-            const int lim = left < static_cast<uint64_t>(kF64Steps) ? static_cast<int>(left) : kF64Steps;
+            const int lim = left < static_cast<uint64_t>(steps) ? static_cast<int>(left) : steps;
             const double *nz = L.nz + static_cast<size_t>(buf) * kF64Steps * cols + L.col[p];
             double kd = static_cast<double>(k0);   // exact below 2^53
             bool esc = false;
@@ -208,17 +315,18 @@ __global__ void __launch_bounds__(32 * kF64Warps, 1) plain_f64_kernel(PlainArgs 
         }
         // The next round's increments, one Philox block of one group at a time.  With fewer
         // groups than schedulers the warps beside a group's leave its scheduler's FP64 unit to it.
-        if (warp < groups || groups == kF64Groups || (warp & 3) >= groups) {
+        const int busy = paired ? 2 * groups : groups;   // schedulers with an integrating warp
+        if (warp < busy || groups == kF64Groups || busy >= kF64Groups || (warp & 3) >= busy) {
             double *out = L.nz + static_cast<size_t>(buf ^ 1) * kF64Steps * cols;
             __syncwarp();
             for (;;) {
                 int item = 0;
                 if (lane == 0) item = atomicAdd(&sh_ticket, 1);
                 item = __shfl_sync(0xFFFFFFFFu, item, 0);
-                if (item >= groups * kF64Blocks) break;
+                if (item >= groups * blocks) break;
                 const int q = 32 * (item % groups) + lane, b = item / groups;
                 if (q < cnt) {
-                    const uint64_t blk = L.blk[q] + (L.col[q] >= 0 ? kF64Blocks : 0) + b;
+                    const uint64_t blk = L.blk[q] + (L.col[q] >= 0 ? blocks : 0) + b;
                     const uint64_t gid = a.traj0 + first + L.idx[q];
                     const uint4 x = philox4x32_10(make_uint4(lo32(blk), hi32(blk), lo32(gid), hi32(gid)),
                                                   a.key0, a.key1);

@@ -48,3 +48,12 @@ def test_step_budgets(cap):
 def test_options(base, over):
     same, esc = _agree(workloads.scaled(base, **over), 2000, 77, traj0=2**32 - 100)
     assert same >= 0.999 and esc > 0.0
+
+
+@pytest.mark.parametrize("over", [dict(), dict(integrator="heun"), dict(nu=0.05), dict(nu=0.05, integrator="heun"),
+                                  dict(sin_amp=0.7), dict(max_steps=29)])
+@pytest.mark.parametrize("n", [152 * 32 + 7, 152 * 64 - 1, 152 * 70])
+def test_underdamped_pairs(over, n):
+    """Two groups per CTA, each integrated by two warps, and three groups, by one each."""
+    same, _ = _agree(workloads.scaled(UNDER, **over), n, 9)
+    assert same >= 0.999
