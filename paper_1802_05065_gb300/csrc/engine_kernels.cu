@@ -970,7 +970,6 @@ __device__ __forceinline__ void tail_integrate(const EngineDev &E, int group, in
     set_idle(L);
     L.c_lo = 0u;
     if (T.slot >= 0) resume_from(L, E, T.slot, T);
-    int n_active = L.slot >= 0 ? 1 : 0;
     float gs, gsl;   // Heun's bias line; an Euler step finds its bias in the noise
     bias_line(fmaf(L.nudt, L.Jf, L.gb), L.nudt, L.dt, gs, gsl);
     const float *end = noise + kTailRing * kNoiseBlock<H>, *cur = noise;   // this block's noise
@@ -978,7 +977,7 @@ __device__ __forceinline__ void tail_integrate(const EngineDev &E, int group, in
     group_barrier(group);
 #pragma unroll
     for (int h = 0; h < kBlockPhilox; ++h) calls[h].load(cur, lane, h);
-    int b = 0, b_count = 0, left = kTailChunk;   // blocks done, blocks counted, blocks left of the chunk
+    int b = 0, left = kTailChunk;   // blocks done, blocks left of the chunk
     for (int parity = 0;;) {
         if constexpr (R && H == kHeun) bias_line(fmaf(L.nudt, L.Jf, L.gb), L.nudt, L.dt, gs, gsl);
         const float *next = cur + kNoiseBlock<H> == end ? noise : cur + kNoiseBlock<H>;
@@ -993,10 +992,9 @@ __device__ __forceinline__ void tail_integrate(const EngineDev &E, int group, in
         if constexpr (R) L.Jf += static_cast<float>(kBlockSteps);
         L.budget -= 1u;
         ++b;
-        bool over = false;
-        if (__any_sync(kFull, mx >= L.hb || L.budget == 0u || L.r < -kPiF)) {
-            useful += static_cast<unsigned long long>(kBlockSteps) * static_cast<unsigned>(n_active * (b - b_count));
-            b_count = b;
+        // Each lane sees to its own event: nothing in here needs the warp, and the vote that
+        // run_blocks takes would hold up the chain at every block.
+        if (mx >= L.hb || L.budget == 0u || L.r < -kPiF) {
             if (mx >= L.hb) {
                 L.r = r0;
                 L.v = v0;
@@ -1010,29 +1008,27 @@ __device__ __forceinline__ void tail_integrate(const EngineDev &E, int group, in
                 }
             }
             if (L.r < -kPiF) wrap_down(L, E);
-            if (L.slot >= 0 && L.c_lo == 0u) L.c_hi += 1u;   // 2^32-block carry
+            if (L.c_lo == 0u) L.c_hi += 1u;   // 2^32-block carry
             if (L.slot >= 0 && (L.esc >= 0 || L.budget == 0u)) {
                 bool escaped = false;
                 unsigned long long k = 0ull;
                 if (finished(L, E, 0u, escaped, k, useful)) {
+                    useful += static_cast<unsigned long long>(kBlockSteps) * static_cast<unsigned>(b);
                     T.fin = escaped ? kTailEscaped : kTailCensored;
                     T.c_lo = static_cast<unsigned>(k);
                     T.c_hi = static_cast<unsigned>(k >> 32);
                     if (escaped) ++n_esc;
                     else ++n_cens;
                     set_idle(L);
-                    n_active = 0;
                 }
-            } else if (L.slot < 0) {
-                L.budget = 0xFFFFFFFFu;
             }
-            over = !__any_sync(kFull, n_active > 0);
             if constexpr (!R && H == kHeun) bias_line(fmaf(L.nudt, L.Jf, L.gb), L.nudt, L.dt, gs, gsl);
         }
         cur = next;
-        if (--left == 0 || b == round || over) {
+        if (--left == 0 || b == round) {
             // Every warp of the group passes the same barriers: the verdict on a chunk lies in the
             // slot of its parity, written again only after the barrier that follows.
+            const bool over = !__any_sync(kFull, L.slot >= 0);
             if (lane == 0) sh.stop[parity][group] = over ? 1 : 0;
             group_barrier(group);
             if (over || b == round) break;
@@ -1040,7 +1036,7 @@ __device__ __forceinline__ void tail_integrate(const EngineDev &E, int group, in
             left = kTailChunk;
         }
     }
-    useful += static_cast<unsigned long long>(kBlockSteps) * static_cast<unsigned>(n_active * (b - b_count));
+    if (L.slot >= 0) useful += static_cast<unsigned long long>(kBlockSteps) * static_cast<unsigned>(b);
     if (L.slot >= 0) {
         T.r = L.r;
         T.v = L.v;
