@@ -21,9 +21,8 @@ time.
 
 Further fields of the one JSON line: `roofline` (XU-pipe bound of the resident kernel, with the
 issue bound at the measured instructions per step; ncu traffic per launch), `e2e` (a fresh
-engine driven through the C ABI from host memory), `fp64_equal_accuracy` (the plain
-one-trajectory-per-thread FP64 kernel against the FP32 engine on one point: the same trajectory
-ids, and both to the same relative standard error), `heun` (the same sweep with the stochastic
+engine driven through the C ABI from host memory), `fp64_equal_accuracy` (the FP64
+kernel against the FP32 engine on one point: the same trajectory ids, and both to the same relative standard error), `heun` (the same sweep with the stochastic
 Heun integrator), `other_workloads` (the ramp sweep, the 256-set uneven batch, the Fig. 10b
 junction, time to solution against N_r), `autotune`, `serving` (Poisson request streams at the
 specified rate and at 0.9x / 0.5x capacity: offered load, p50 / p99 latency and slowdown, FP32
@@ -269,8 +268,8 @@ def roofline_model(n_sm: int, f_mhz: float):
 
 
 def fp64_equal_accuracy(pkg, torch, dev, point, block, T, bps):
-    """The FP32 persistent engine against the plain one-trajectory-per-thread FP64 kernel on one
-    point (Alg. 1 structure, every operation in double precision), at equal accuracy:
+    """The FP32 persistent engine against the FP64 kernel (Alg. 1, every operation in double
+    precision and rounded as written) on one point, at equal accuracy:
       same_ids: both integrate the same 2^20 trajectory ids of the same seed, so their means
                 carry the same statistical error; time to solution, trajectory-steps/s, mean and
                 SEM of each, and the per-trajectory difference of the escape times (FP32 - FP64);
@@ -530,15 +529,18 @@ def run_ours(args):
         el_max = allreduce(el, "max")
         st_all = allreduce(cc["useful_steps"])
         maxr = 256
-        h2d = (12 * (176 + 96) + args.steps * maxr * 4 * 3) / args.steps
-        d2h = (args.steps * (maxr * 96 + 32) + hbytes) / args.steps
+        # up: constants and control block per request, then the lists of each iteration; down: the
+        # control block of every request in a slot and the counters, which the scan kernel writes
+        # to pinned memory each iteration, and the histograms
+        h2d = (len(pts) * (280 + 112) + args.steps * 4 * (24 + 10 * maxr)) / args.steps
+        d2h = (args.steps * (len(pts) * 112 + 32) + hbytes) / args.steps
         e2e = {"value": st_all / el_max, "unit": UNIT, "h2d_bytes_per_step": int(h2d),
                "d2h_bytes_per_step": int(d2h),
                "escapes_per_s": allreduce(cc["escapes"]) / el_max}
         eng2.close()
 
-    # the plain one-trajectory-per-thread FP64 kernel (Alg. 1 structure, paper-literal FP64)
-    # against the FP32 engine at equal accuracy on the gamma = 0.9, D = 0.2 point
+    # the FP64 kernel (Alg. 1 in double precision) against the FP32 engine at equal accuracy on the
+    # gamma = 0.9, D = 0.2 point
     fp64 = None
     if not args.no_fp64 and rank == 0:
         fp64 = fp64_equal_accuracy(pkg, torch, local, pts[11], args.block, args.traj_per_thread,

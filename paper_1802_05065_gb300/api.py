@@ -23,7 +23,7 @@ def current_stream(device=None) -> int:
 
 def run_plain(d: dict, n: int, seed: int, traj0: int = 0, device=None, **over):
     """Escape steps (int64 device tensor, -1 = censored) of trajectories traj0..traj0+n-1 from
-    the one-trajectory-per-thread kernel (FP64 or FP32 per d['precision'])."""
+    the plain kernels (FP64 or FP32 per d['precision'])."""
     torch = _torch()
     p = _lib.params_from(d, **over)
     dev = torch.device(device) if device is not None else torch.device("cuda")

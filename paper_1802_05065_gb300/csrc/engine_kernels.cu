@@ -193,7 +193,7 @@ struct CtaView {
     unsigned *share;             // blocks of the launch every warp runs before it takes from the pool
     int *tail;                   // 1: the CTA's warps meet to run its last trajectories together
     // Groups of 32 lanes the CTA can run that way (0: it never does).  In shared memory like the rest: a
-    // register held through run_blocks costs its loop 1 % (1188 -> 1199 Gstep/s over the 20-point sweep).
+    // register held through run_blocks costs its loop 1 % (1188 -> 1199 Gstep/s over the 12-point sweep).
     const int *tail_groups;
     const int *act_count;        // the launch's lists and flags, read once: claimable slots per kind,
     const int *flags;            // {strict caps, warps of the CTA that claim}
@@ -596,7 +596,7 @@ __device__ __forceinline__ bool more(const CtaView &V, unsigned &limit) {
 
 // Until the blocks are used up, the warp's trajectories are, or some of its lanes find no more work:
 // then the caller looks whether the CTA has run dry.  (With that look in here the loop of a full CTA
-// took 1 % more time: 1176 -> 1188 Gstep/s over the 20-point sweep.)
+// took 1 % more time: 1176 -> 1188 Gstep/s over the 12-point sweep.)
 template <int M, int H, int R, int T>
 __device__ __forceinline__ unsigned run_blocks(Lane (&L)[T], const EngineDev &E, const CtaView &V, unsigned b,
                                                int &n_active,

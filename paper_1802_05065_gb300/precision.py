@@ -1,15 +1,14 @@
 """Error of the single-precision engine against the double-precision kernel, per workload.
 
-The FP32 engine and the plain one-trajectory-per-thread FP64 kernel (the arithmetic of Alg. 1 /
-Alg. 3 in double precision) integrate the same trajectory ids of the same seed.  The FP32
+The FP32 engine and the FP64 kernel (the arithmetic of Alg. 1 / Alg. 3 in double precision) integrate the same trajectory ids of the same seed.  The FP32
 uniform is the FP64 one rounded to 23 bits, so both paths see nearly the same noise and the
 per-trajectory difference of the result (escape time or switching bias) isolates the error of
 single precision.  Reported per case: both means and standard errors, the mean paired difference
 and its standard error, the difference of means in combined standard errors, and the
 two-sample Kolmogorov-Smirnov p-value of the two result distributions.
 
-Cost: the FP64 kernel advances one trajectory per thread at ~3e5 steps/s on a GB300, so a case
-takes (trajectory length / 3e5) seconds whatever its trajectory count up to a few thousand.
+Cost: the FP64 kernel advances a trajectory at ~1e6 steps/s on a GB300, so a case takes
+(trajectory length / 1e6) seconds whatever its trajectory count up to ~10 000.
 The report over every config is `python bench.py --precision-report`.
 """
 from __future__ import annotations
