@@ -1246,7 +1246,11 @@ __device__ __noinline__ void tail_run(const EngineDev &E, int *held, int groups,
     if (lane == 0) E.warp_kind[gtid >> 5] = warp < groups ? sh.kind[warp] : -1;
 }
 
-template <int T>
+// kTail: with the packed last trajectories.  Their named barriers count as all 16 of a CTA, which an SM
+// has for four CTAs: small CTAs, which run no groups, get the kernel without (one to four warps: 16, 10,
+// 6 and 5 CTAs per SM; the sweep at 32 / 64 / 128 threads with four: 493 / 821 / 1012 Gstep/s, so:
+// 986 / 1034 / 1039).
+template <int T, bool kTail>
 __global__ void __launch_bounds__(T == 1 ? 640 : 256, 1) engine_chunk_kernel(const __grid_constant__ EngineDev E) {
     const unsigned nthreads = gridDim.x * blockDim.x;
     const unsigned gtid = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1262,7 +1266,7 @@ __global__ void __launch_bounds__(T == 1 ? 640 : 256, 1) engine_chunk_kernel(con
     __shared__ unsigned sh_chunk, sh_share;
     __shared__ int sh_warp_act[32], sh_warp_knd[32], sh_tail, sh_done, sh_act_count[kNumKinds], sh_flags[2], sh_tail_groups;
     // while caps are enforced the lanes that idle are meant to
-    const int tail_groups = *E.strict != 0 ? 0 : tail_groups_of(T, static_cast<int>(blockDim.x >> 5));
+    const int tail_groups = !kTail || *E.strict != 0 ? 0 : tail_groups_of(T, static_cast<int>(blockDim.x >> 5));
     const CtaView V{sh_ok, sh_held, sh_budget, sh_res_slot, sh_res_cnt, sh_res_base, sh_started, &sh_pool,
                     sh_warp_act, sh_warp_knd, &sh_share, &sh_tail, &sh_tail_groups, sh_act_count, sh_flags};
     for (int s = threadIdx.x; s < E.max_requests; s += blockDim.x) {
@@ -1371,7 +1375,7 @@ __global__ void __launch_bounds__(T == 1 ? 640 : 256, 1) engine_chunk_kernel(con
             work |= (ok & 3u) != 0u;
         }
         work = __syncthreads_or(work) != 0;
-        if (T == 1 && tail_groups > 0 && !work && thinned_out(V)) {
+        if (kTail && tail_groups > 0 && !work && thinned_out(V)) {
             dry = true;
             if (threadIdx.x == 0) sh_tail = 1;
         }
@@ -1402,10 +1406,10 @@ __global__ void __launch_bounds__(T == 1 ? 640 : 256, 1) engine_chunk_kernel(con
                 break;
 #undef FPT_KIND_CASE
             }
-            if (T == 1 && !__all_sync(kFull, L[0].slot >= 0)) look_dry(L, E, V, kind);
+            if (kTail && !__all_sync(kFull, L[0].slot >= 0)) look_dry(L, E, V, kind);
             if (!__any_sync(kFull, n_active > 0)) kind = -1;
         }
-        if constexpr (T == 1) {
+        if constexpr (kTail) {
             if (tail_groups > 0) {
                 // the blocks left in this launch, after the furthest of the warps with trajectories
                 if (lane == 0 && kind >= 0) atomicMax(&sh_done, static_cast<int>(b));
@@ -1769,12 +1773,13 @@ __global__ void engine_scan_kernel(EngineDev E, SlotCtl *h_ctl, unsigned long lo
 
 cudaError_t launch_engine_chunk(const EngineDev &E, int T, unsigned grid, unsigned block,
                                 cudaStream_t s) {
-    if (T == 1) {
-        const size_t shared = tail_shared_bytes(static_cast<int>(block / 32));
-        engine_chunk_kernel<1><<<grid, block, shared, s>>>(E);
-    } else {
-        engine_chunk_kernel<2><<<grid, block, 0, s>>>(E);
-    }
+    const size_t shared = tail_shared_bytes(static_cast<int>(block / 32));
+    if (T != 1)
+        engine_chunk_kernel<2, false><<<grid, block, 0, s>>>(E);
+    else if (shared == 0)
+        engine_chunk_kernel<1, false><<<grid, block, 0, s>>>(E);
+    else
+        engine_chunk_kernel<1, true><<<grid, block, shared, s>>>(E);
     return cudaGetLastError();
 }
 
@@ -1829,16 +1834,15 @@ cudaError_t launch_engine_scan(const EngineDev &E, SlotCtl *h_ctl, unsigned long
 }
 
 cudaError_t engine_chunk_occupancy(int T, int block, int *blocks_per_sm) {
-    if (T == 1) {
-        // every engine asks before its first launch, so the kernel's shared-memory limit is set
-        const cudaError_t e = cudaFuncSetAttribute(engine_chunk_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   static_cast<int>(tail_shared_bytes(640 / 32)));
-        if (e != cudaSuccess) return e;
-        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, engine_chunk_kernel<1>, block,
-                                                             tail_shared_bytes(block / 32));
-    }
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, engine_chunk_kernel<2>,
-                                                         block, 0);
+    const size_t shared = tail_shared_bytes(block / 32);
+    if (T != 1) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, engine_chunk_kernel<2, false>, block, 0);
+    if (shared == 0)
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, engine_chunk_kernel<1, false>, block, 0);
+    // every engine asks before its first launch, so the kernel's shared-memory limit is set
+    const cudaError_t e = cudaFuncSetAttribute(engine_chunk_kernel<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               static_cast<int>(tail_shared_bytes(640 / 32)));
+    if (e != cudaSuccess) return e;
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, engine_chunk_kernel<1, true>, block, shared);
 }
 
 }  // namespace fpt

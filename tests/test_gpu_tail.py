@@ -60,6 +60,13 @@ def test_cta_sizes(threads):
     assert (k == _plain(OVER, 30011, 8)).all()
 
 
+@pytest.mark.parametrize("threads,ctas", [(32, 16), (64, 10), (96, 6), (128, 5), (256, 2), (640, 1)])
+def test_ctas_per_sm(threads, ctas):
+    """What registers (20 warps of 96) and static shared memory allow: the groups cost no CTA."""
+    from paper_1802_05065_gb300 import _lib
+    assert _lib.engine_occupancy(1, threads) == ctas
+
+
 def test_kinds_mixed():
     reqs = [(d, 700 + 301 * i, 50 + i) for i, d in enumerate(KINDS)]
     for k, (d, n, s) in zip(_run(reqs, chunk_steps=4096), reqs):
