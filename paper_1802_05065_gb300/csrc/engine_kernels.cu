@@ -60,6 +60,7 @@ enum : unsigned {
     kChkTraj = 5,      // trajectory index outside [0, n_traj)
     kChkPark = 6,      // suspended-trajectory ring index outside [0, park_cap)
     kChkKind = 7,      // kind outside [0, kNumKinds)
+    kChkReservoir = 8,   // a warp goes on to the packed last trajectories with ids in its reservoir
 };
 #ifdef FPT_CHECK
 __device__ __forceinline__ bool checked(const EngineDev &E, bool ok, unsigned bit) {
@@ -557,7 +558,9 @@ __device__ __forceinline__ bool thinned_out(const CtaView &V) {
 // This warp's lanes after an event, for the CTA's view, and whether the CTA has run dry
 // (warp-collective): nothing left to claim or resume in any listed request, no reservoir, and
 // trajectories thinned out.  Then the warps are called together (V.tail); the exact counts are taken
-// when they have met.
+// when they have met.  Flags before reservoirs: refill fills a warp's reservoir before it clears the
+// flag.  A claim can still be under way here whose ids nobody sees yet, so a warp gives back what its
+// reservoir holds on its way to the meeting.
 template <int T>
 __device__ __forceinline__ void look_dry(Lane (&L)[T], const EngineDev &E, const CtaView &V, int kind) {
     if constexpr (T == 1) {
@@ -570,10 +573,11 @@ __device__ __forceinline__ void look_dry(Lane (&L)[T], const EngineDev &E, const
         }
         __syncwarp();
         if (!thinned_out(V)) return;
-        bool work = lane < warps && vload(V.res_cnt[lane]) > 0;
+        bool work = false;
         for (int k = 0; k < kNumKinds; ++k)
             for (int j = lane; j < V.act_count[k]; j += 32)
                 work |= (vload(V.ok[E.act_list[k * E.max_requests + j]]) & 3u) != 0u;
+        work |= lane < warps && vload(V.res_cnt[lane]) > 0;
         if (!__any_sync(kFull, work) && lane == 0) *V.tail = 1;
     }
 }
@@ -1409,6 +1413,36 @@ __global__ void __launch_bounds__(T == 1 ? 640 : 256, 1) engine_chunk_kernel(con
             if (kTail && !__all_sync(kFull, L[0].slot >= 0)) look_dry(L, E, V, kind);
             if (!__any_sync(kFull, n_active > 0)) kind = -1;
         }
+        // Ids left in this warp's reservoir go back to their request as suspended trajectories that
+        // have not started (state r0, v0, w0 at step 0: resuming one is starting it).  The CTA's
+        // budget kept the ring's room for them.  Before the meeting: a warp that goes on from there
+        // finds the claim flags cleared, so no reservoir is filled again, and tail_run ends the launch.
+        {
+            __syncwarp();
+            const int wl = static_cast<int>(threadIdx.x >> 5);
+            const int rs = sh_res_slot[wl], rc = sh_res_cnt[wl];
+            if (rs >= 0 && rc > 0 && checked(E, rs < E.max_requests, kChkSlot)) {
+                SlotCtl *C = E.ctl + rs;
+                const SlotDev *S = E.slots + rs;
+                for (int j = lane; j < rc; j += 32) {
+                    const unsigned long long gid = S->traj_offset + sh_res_base[wl] + static_cast<unsigned long long>(j);
+                    const int used = atomicAdd(&C->park_used, 1);
+                    checked(E, used < static_cast<int>(S->park_cap), kChkPark);   // the budget's invariant
+                    const unsigned pi = atomicAdd(&C->park_tail, 1u);
+                    if (!checked(E, pi % S->park_cap < S->park_cap, kChkPark)) continue;
+                    ParkEntry &P = S->park[pi % S->park_cap];
+                    P.r = S->r0;
+                    P.v = S->v0;
+                    P.w = S->w0;
+                    P.c_lo = P.c_hi = 0u;
+                    P.gid_lo = static_cast<unsigned>(gid);
+                    P.gid_hi = static_cast<unsigned>(gid >> 32);
+                    P.pad = 0;
+                }
+            }
+            __syncwarp();
+            if (lane == 0) sh_res_cnt[wl] = 0;
+        }
         if constexpr (kTail) {
             if (tail_groups > 0) {
                 // the blocks left in this launch, after the furthest of the warps with trajectories
@@ -1417,6 +1451,7 @@ __global__ void __launch_bounds__(T == 1 ? 640 : 256, 1) engine_chunk_kernel(con
                 if (sh_tail != 0) {
                     const int groups = tail_pack(L, kind);
                     if (groups <= tail_groups) {
+                        checked(E, vload(sh_res_cnt[threadIdx.x >> 5]) == 0, kChkReservoir);
                         if (lane == 0) E.warp_cursor[warp] = cursor;
                         add_counters(E, useful, n_esc, n_cens);
                         const unsigned done = static_cast<unsigned>(sh_done);
@@ -1466,33 +1501,6 @@ __global__ void __launch_bounds__(T == 1 ? 640 : 256, 1) engine_chunk_kernel(con
         atomicSub(&C->inflight, 1);
         L[t].slot = -1;
         --n_active;
-    }
-    // Ids left in this warp's reservoir go back to their request as suspended trajectories that
-    // have not started (state r0, v0, w0 at step 0: resuming one is starting it).  The CTA's
-    // budget kept the ring's room for them.
-    {
-        __syncwarp();
-        const int wl = static_cast<int>(threadIdx.x >> 5);
-        const int rs = sh_res_slot[wl], rc = sh_res_cnt[wl];
-        if (rs >= 0 && rc > 0 && checked(E, rs < E.max_requests, kChkSlot)) {
-            SlotCtl *C = E.ctl + rs;
-            const SlotDev *S = E.slots + rs;
-            for (int j = lane; j < rc; j += 32) {
-                const unsigned long long gid = S->traj_offset + sh_res_base[wl] + static_cast<unsigned long long>(j);
-                const int used = atomicAdd(&C->park_used, 1);
-                checked(E, used < static_cast<int>(S->park_cap), kChkPark);   // the budget's invariant
-                const unsigned pi = atomicAdd(&C->park_tail, 1u);
-                if (!checked(E, pi % S->park_cap < S->park_cap, kChkPark)) continue;
-                ParkEntry &P = S->park[pi % S->park_cap];
-                P.r = S->r0;
-                P.v = S->v0;
-                P.w = S->w0;
-                P.c_lo = P.c_hi = 0u;
-                P.gid_lo = static_cast<unsigned>(gid);
-                P.gid_hi = static_cast<unsigned>(gid >> 32);
-                P.pad = 0;
-            }
-        }
     }
     if (!__any_sync(kFull, n_active > 0)) kind = -1;
 #pragma unroll
