@@ -156,6 +156,16 @@ FPT_HD inline uint32_t claim_blocks_for(double ids, uint32_t stop_block, uint32_
     return blocks + 2.0 < 4.0e9 ? static_cast<uint32_t>(blocks + 2.0) : 0u;
 }
 
+// Rounds of a CTA's last trajectories: blocks of the next one, at most `most`, which doubles after each
+// round that needed no packing.  Capped, because a launch without an end (fpt_run_noalloc's) takes more
+// than 2^31 blocks of a trajectory that hardly ever escapes and a round's blocks are counted in an int; the
+// meeting after 2^20 blocks (~0.3 s) costs nothing.
+constexpr unsigned kRoundBlocks = 256, kRoundBlocksMax = 1u << 20;
+FPT_HD inline int round_blocks(uint64_t blocks, unsigned most) {
+    return static_cast<int>(blocks < most ? blocks : most);
+}
+FPT_HD inline unsigned longer_round(unsigned most) { return most < kRoundBlocksMax ? 2u * most : most; }
+
 struct LaneSoA {
     float *r, *v;
     int *w, *slot;

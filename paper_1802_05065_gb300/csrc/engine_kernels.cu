@@ -756,7 +756,6 @@ constexpr int kTailGroupsMax = 5;       // a quarter of the warps: one scheduler
 constexpr int kTailMakers = 3;          // noise warps per group
 constexpr int kTailChunk = 3;           // blocks per chunk, one for each of them
 constexpr int kTailRing = 3 * kTailChunk;                     // blocks in a group's ring
-constexpr int kRoundBlocks = 256;
 // Floats of one block of a group.  Euler: the 16 addends of the steps (noise and bias, formed by
 // the noise warps: an operation and half a load per step less in the chain's warp); Heun: 8 radii
 // and 16 cosines / sines, as its two stages take different biases.
@@ -1154,7 +1153,7 @@ __device__ __noinline__ void tail_run(const EngineDev &E, int *held, int groups,
     const int warp = static_cast<int>(threadIdx.x >> 5), lane = threadIdx.x & 31;
     const int warps = static_cast<int>(blockDim.x >> 5);
     const unsigned gtid = blockIdx.x * blockDim.x + threadIdx.x;
-    unsigned most = kRoundBlocks;   // doubled after each round that needed no packing
+    unsigned most = kRoundBlocks;
     while (blocks > 0 && groups > 0) {
         // Roles.  Euler: warp 4 g integrates group g (scheduler 0), the warps of the other
         // schedulers make noise, the m-th of them for group m mod groups.  A Heun step's two sines
@@ -1169,7 +1168,7 @@ __device__ __noinline__ void tail_run(const EngineDev &E, int *held, int groups,
         else m = (warp & 1) ? warp >> 1 : (warps >> 1) + (warp >> 1) - groups;
         const int group = integrates ? warp / spread : m % groups;
         const int rank = m / groups;
-        const int round = blocks < most ? static_cast<int>(blocks) : static_cast<int>(most);
+        const int round = round_blocks(blocks, most);
         if (integrates) {
             if constexpr (K >= 0) tail_integrate<(K & 1), ((K >> 1) & 1), (K >> 2)>(E, group, round);
             else switch (sh.kind[group]) {
@@ -1210,7 +1209,7 @@ __device__ __noinline__ void tail_run(const EngineDev &E, int *held, int groups,
         }
         __syncthreads();
         if (fewer == groups) {
-            most *= 2u;
+            most = longer_round(most);
             continue;
         }
         most = kRoundBlocks;
