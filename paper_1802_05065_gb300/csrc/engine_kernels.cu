@@ -61,6 +61,7 @@ enum : unsigned {
     kChkPark = 6,      // suspended-trajectory ring index outside [0, park_cap)
     kChkKind = 7,      // kind outside [0, kNumKinds)
     kChkReservoir = 8,   // a warp goes on to the packed last trajectories with ids in its reservoir
+    kChkDry = 9,       // a warp skips its blocks for a meeting that is not called
 };
 #ifdef FPT_CHECK
 __device__ __forceinline__ bool checked(const EngineDev &E, bool ok, unsigned bit) {
@@ -1364,8 +1365,9 @@ __global__ void __launch_bounds__(T == 1 ? 640 : 256, 1) engine_chunk_kernel(con
             sh_warp_knd[threadIdx.x >> 5] = kind < 0 ? 0 : kind;
         }
     }
-    // Dry from the start?  The queue heads as they are after this CTA's first claims; all warps see
-    // the same, so they go straight to the meeting.
+    // Dry from the start?  The queue heads as they are after this CTA's first claims.  One warp decides
+    // for all, between two barriers: the counts it reads change as soon as a warp runs on.  Then they go
+    // straight to the meeting.
     bool dry = false;
     {
         bool work = false;
@@ -1378,9 +1380,9 @@ __global__ void __launch_bounds__(T == 1 ? 640 : 256, 1) engine_chunk_kernel(con
             work |= (ok & 3u) != 0u;
         }
         work = __syncthreads_or(work) != 0;
-        if (kTail && tail_groups > 0 && !work && thinned_out(V)) {
-            dry = true;
-            if (threadIdx.x == 0) sh_tail = 1;
+        if (kTail && tail_groups > 0 && !work) {
+            dry = __syncthreads_or(threadIdx.x < 32 && thinned_out(V)) != 0;
+            if (dry && threadIdx.x == 0) sh_tail = 1;
         }
     }
     unsigned limit = 0;
@@ -1447,6 +1449,7 @@ __global__ void __launch_bounds__(T == 1 ? 640 : 256, 1) engine_chunk_kernel(con
                 // the blocks left in this launch, after the furthest of the warps with trajectories
                 if (lane == 0 && kind >= 0) atomicMax(&sh_done, static_cast<int>(b));
                 __syncthreads();
+                checked(E, !dry || sh_tail != 0, kChkDry);
                 if (sh_tail != 0) {
                     const int groups = tail_pack(L, kind);
                     if (groups <= tail_groups) {

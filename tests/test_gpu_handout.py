@@ -3,7 +3,8 @@ their reservoirs hold.  Stop-rule requests of trajectories of a few to a hundred
 kinds at once: warps claim ahead, the hand-out limit is passed and raised again and again, and CTAs are
 always thin.  (A million trajectories of a few blocks with a 0.3 % rule: 3 to 9 warps per run hold ids
 when their CTA meets.)  Every request completes, its prefix holds exactly the escape steps of the plain
-kernel, and the bounds-checked build finds no reservoir after the meeting."""
+kernel, and the bounds-checked build finds no reservoir after the meeting, nor a warp that waits for a
+meeting nobody called when CTAs start a launch with nothing left to claim."""
 import os
 import subprocess
 import sys
@@ -43,11 +44,12 @@ def test_every_id_of_the_prefix(problems, chunk):
     run_requests(problems, chunk, range(6))
 
 
-def test_checked_build():
+@pytest.mark.parametrize("problem,chunks", [("BLOCKS", (1024, 4096, 16384)), ("LONGER", (64, 256, 1024))])
+def test_checked_build(problem, chunks):
     from paper_1802_05065_gb300 import build as b
     b.build()
-    code = """from tests.test_gpu_handout import *
-for chunk in (1024, 4096, 16384): run_requests([BLOCKS], chunk, (1, 2, 3))"""
+    code = f"""from tests.test_gpu_handout import *
+for chunk in {chunks}: run_requests([{problem}], chunk, (1, 2, 3))"""
     p = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, cwd=ROOT, timeout=900,
                        env=dict(os.environ, FPT_LIBRARY=b.LIB_CHECK))
     assert p.returncode == 0, p.stderr[-3000:]
