@@ -390,7 +390,7 @@ fpt_status admit(fpt_engine *e) {
             R.restore.clear();
             R.restore.shrink_to_fit();
         } else if (R.params.stop_rse > 0.0) {
-            C.claim_blocks = claim_blocks_for(1.0 / (R.params.stop_rse * R.params.stop_rse), R.stop_block, 0);
+            C.claim_blocks = claim_blocks_for(1.0 / (R.params.stop_rse * R.params.stop_rse), R.stop_block, 0, e->sms);
         }
         R.claim_end0 = claim_end(R.n_traj, R.stop_block, C.claim_blocks);
         C.state = kSlotActive;
@@ -858,6 +858,7 @@ fpt_status create_impl(const fpt_engine_config *cfg_in, fpt_engine *e) {
     d.counters = e->d_counters;
     d.chunk_blocks = e->chunk_blocks;
     d.max_requests = R;
+    d.sms = e->sms;
     d.n_lanes = e->lanes;
     CK(cudaStreamSynchronize(e->stream));
     if (cfg.use_graph)

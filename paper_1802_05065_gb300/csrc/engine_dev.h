@@ -146,9 +146,9 @@ FPT_HD inline uint64_t claim_end(uint64_t n_traj, uint32_t stop_block, uint32_t 
 
 // Blocks to hand out when `prefix` of them are folded and the rule needs `ids` trajectories in all:
 // a quarter more than that, half as much again as is folded, and never fewer ids ahead than two
-// warps per SM, which run no slower than one.
-FPT_HD inline uint32_t claim_blocks_for(double ids, uint32_t stop_block, uint32_t prefix) {
-    const double B = stop_block, p = prefix, ahead = 64.0 * 152.0;
+// warps per SM, which run no slower than one (`sms`: the engine's device; a whole GB300 has 152).
+FPT_HD inline uint32_t claim_blocks_for(double ids, uint32_t stop_block, uint32_t prefix, int sms = 152) {
+    const double B = stop_block, p = prefix, ahead = 64.0 * sms;
     double blocks = 1.25 * ids / B;
     if (!(blocks < 4.0e9)) return 0;   // also a NaN: no limit
     if (blocks < 1.5 * p) blocks = 1.5 * p;
@@ -194,6 +194,7 @@ struct EngineDev {
     unsigned long long *counters;
     unsigned int chunk_blocks;   // blocks per warp of a full launch
     int max_requests;
+    int sms;                // SMs of the device
     unsigned int n_lanes;   // threads x trajectories per thread (lane state entries)
 };
 

@@ -1767,7 +1767,7 @@ __global__ void engine_scan_kernel(EngineDev E, SlotCtl *h_ctl, unsigned long lo
             C->prefix = p;
             if (finished) C->state = kSlotFinished;
             else if (C->claim_blocks != 0 && p > first) {
-                const unsigned claim = claim_blocks_for(need, S->stop_block, p);
+                const unsigned claim = claim_blocks_for(need, S->stop_block, p, E.sms);
                 if (claim == 0 || claim > C->claim_blocks) C->claim_blocks = claim;
             }
         }

@@ -667,10 +667,14 @@ cudaError_t launch_plain_f64(const PlainArgs &a, cudaStream_t s) {
 }
 
 cudaError_t launch_plain_f32(const PlainArgs &a, cudaStream_t s) {
-    // CTAs of one warp while every warp can have a scheduler to itself (152 SMs x 4), so that few
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    // CTAs of one warp while every warp can have a scheduler to itself (four per SM), so that few
     // trajectories spread over all of them; then of two, so that a CTA waits for 64 trajectories
     // rather than 256 before its place is free (2^18 trajectories: 56 -> 55 ms).
-    const unsigned block = a.n <= 32 * 4 * 152 ? 32 : 64;
+    const unsigned block = a.n <= 32ull * 4 * static_cast<unsigned>(sms) ? 32 : 64;
     const unsigned grid = grid_for(a.n, block);
     switch (a.kind) {
 #define FPT_KIND_CASE(M_, H_, R_) \

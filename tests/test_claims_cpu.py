@@ -50,3 +50,31 @@ def test_claims(tmp_path):
         else:
             assert prefix < b and b * block >= min(ids, 2.0**63) and end == min(n, b * block)
             assert b * block <= 1.25 * ids + 1.5 * prefix * block + prefix * block + 64 * 152 + 3 * block
+
+
+SMS_PROGRAM = r"""
+#include <cstdio>
+#include "engine_dev.h"
+int main() {
+    for (int sms : {1, 76, 132, 148, 152, 160})
+        for (unsigned prefix : {0u, 3u, 1000u})
+            std::printf("%d %u %u\n", sms, prefix, fpt::claim_blocks_for(0.0, 64, prefix, sms));
+    return 0;
+}
+"""
+
+
+def test_look_ahead_follows_the_device(tmp_path):
+    """Two warps per SM ahead of the folded prefix, whatever number of SMs the engine's device has."""
+    nvcc = _nvcc()
+    if nvcc is None:
+        pytest.skip("nvcc not installed")
+    src, exe = tmp_path / "s.cu", tmp_path / "s"
+    src.write_text(SMS_PROGRAM)
+    r = subprocess.run([nvcc, "-O2", "-std=c++17", "-I", CSRC, "-o", str(exe), str(src)], capture_output=True,
+                       text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-3000:]
+    lines = subprocess.run([str(exe)], capture_output=True, text=True).stdout.splitlines()
+    assert len(lines) == 18
+    for sms, prefix, blocks in (map(int, l.split()) for l in lines):
+        assert max(64 * sms, 32 * prefix) <= 64 * (blocks - prefix) <= max(64 * sms, 32 * prefix) + 2 * 64
