@@ -74,3 +74,40 @@ def test_stop_rule_hands_out_what_it_needs():
             r = eng.wait(eng.submit(m.params_from(p), 200_000, 4), 120.0)
             c = eng.counters()
             assert lo <= r.n_used <= c["escapes"] + c["censored"] <= hi, (d, r.n_used, c)
+
+
+def test_release_during_a_read():
+    """One thread copies a finished request's steps while another releases it and runs the next, which
+    would take its buffer: a copy that began gives the first request's steps."""
+    import threading
+    import time
+    import paper_1802_05065_gb300 as m
+    from paper_1802_05065_gb300 import api
+    n, d = 500_001, workloads.scaled(OVER, max_steps=300)
+    want = [api.run_plain(d, n, s).cpu().numpy() for s in range(2)]
+    reads = 0
+    with m.Engine(0, chunk_steps=4096) as eng:
+        p = m.params_from(d, keep_per_traj=1)
+        rid = eng.submit(p, n, 0)
+        eng.wait(rid, 120.0)
+        for i in range(40):
+            got, begun = [], threading.Event()
+
+            def read(rid=rid):
+                begun.set()
+                try:
+                    got.append(eng.per_traj_steps(rid, n))
+                except m.FptError as e:   # the release came first
+                    got.append(e)
+            t = threading.Thread(target=read)
+            t.start()
+            begun.wait()
+            time.sleep(1e-4 * i)   # a copy takes ~1 ms: before, during and after it
+            eng.release(rid)
+            rid = eng.submit(p, n, (i + 1) % 2)
+            eng.wait(rid, 120.0)
+            t.join()
+            if not isinstance(got[0], m.FptError):
+                reads += 1
+                assert (got[0] == want[i % 2]).all()
+    assert reads > 0

@@ -68,3 +68,27 @@ def test_accumulates_and_overlaps():
     torch.cuda.synchronize()
     a.check(3)
     b.check(3)
+
+
+CAPTURE = """
+import torch
+from tests.test_gpu_solo import *
+from tests.test_gpu_solo import _Call
+a = _Call(OVER, 50001, 4)
+g = torch.cuda.CUDAGraph()
+with torch.cuda.graph(g):   # the process's first call of the library
+    a.launch(torch.cuda.current_stream().cuda_stream)
+for _ in range(3):
+    g.replay()
+torch.cuda.synchronize()
+a.check(3)
+"""
+
+
+def test_first_call_inside_a_stream_capture():
+    import os
+    import subprocess
+    import sys
+    p = subprocess.run([sys.executable, "-c", CAPTURE], capture_output=True, text=True, timeout=600,
+                       cwd=os.path.dirname(os.path.dirname(os.path.abspath(__file__))))
+    assert p.returncode == 0, p.stderr[-3000:]
