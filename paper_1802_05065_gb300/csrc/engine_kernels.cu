@@ -285,7 +285,9 @@ __device__ __forceinline__ void emit_warp(const EngineDev &E, int *held, bool fi
 // hardly depends on how many lanes it serves: a warp that starts a trajectory at least every eight
 // blocks takes the escapes of up to kDeferBlocks further blocks together.  Lane::esc holds the step
 // in its block and that block's number modulo kDeferMask + 1.  (Trajectories of 950 steps, 60
-// blocks: 8.4 -> 6.8 ms for 2^22, with the integer bins of hist_bin.)
+// blocks: 8.4 -> 6.8 ms for 2^22, with the integer bins of hist_bin.  Kinds whose trajectories last 10^4
+// steps never wait, but their loop holds the test: ramped Euler at seven warps per SM 40.8 -> 42.6 ns per
+// step, a switching histogram of 30 000 trajectories 43.1 -> 45.)
 constexpr unsigned kDeferBlocks = 5, kDeferMask = 15u;
 constexpr int kDeferShift = 8;
 
@@ -521,9 +523,6 @@ __device__ __forceinline__ int refill(Lane (&L)[T], const EngineDev &E, const Ct
     return total;
 }
 
-// Integrate blocks of kBlockSteps steps with model M, integrator H and bias kind R (constant or
-// ramped) until the warp's share of the launch's blocks is done (`limit`, extended from the
-// CTA's pool) or the whole warp has run out of work.  Returns the next block index.
 // A launch's blocks: each warp first runs (1 - 1/kPoolDiv) of the launch's block count, then
 // takes kGrant blocks at a time from its CTA's pool of the rest, so warps whose lanes had more
 // events (replays, refills) do fewer blocks and the warps of an SM finish together instead of
@@ -599,9 +598,11 @@ __device__ __forceinline__ bool more(const CtaView &V, unsigned &limit) {
     return grant(V, limit);
 }
 
-// Until the blocks are used up, the warp's trajectories are, or some of its lanes find no more work:
-// then the caller looks whether the CTA has run dry.  (With that look in here the loop of a full CTA
-// took 1 % more time: 1176 -> 1188 Gstep/s over the 12-point sweep.)
+// Integrate blocks of kBlockSteps steps with model M, integrator H and bias kind R (constant or
+// ramped) until the warp's share of the launch's blocks is done (`limit`, extended from the
+// CTA's pool), the whole warp has run out of work, or some of its lanes find no more: then the caller
+// looks whether the CTA has run dry.  Returns the next block index.  (With that look in here the loop of
+// a full CTA took 1 % more time: 1176 -> 1188 Gstep/s over the 12-point sweep.)
 template <int M, int H, int R, int T>
 __device__ __forceinline__ unsigned run_blocks(Lane (&L)[T], const EngineDev &E, const CtaView &V, unsigned b,
                                                int &n_active,
@@ -717,9 +718,6 @@ __device__ __forceinline__ unsigned run_blocks(Lane (&L)[T], const EngineDev &E,
     return b;
 }
 
-// One trajectory per thread runs best as one CTA of 640 threads per SM: 20 warps, five per
-// scheduler, at 96 registers (measured against 512, 576, 672 and 768); two per thread as CTAs
-// of up to 256.
 // An idle warp looks for work of any kind, starting from a warp-dependent one; returns the kind
 // it took work of, or -1.
 template <int T>
@@ -752,7 +750,7 @@ __device__ __forceinline__ int seek_work(Lane (&L)[T], const EngineDev &E, const
 // run_blocks, bit for bit.  ns per step at 1 / 2 / 3 / 4 full warps per SM, the plain loop -> this:
 // overdamped Euler 31.5 / 31.5 / 31.5 / 31.5 -> 17.5 / 18.5 / 21.2 / 22.8, underdamped ramped Euler
 // 30.4 / 30.5 / 30.5 / 30.5 -> 12.8 / 17.5 / 21.4 / 23.0, underdamped Heun 40 -> 24 / 25 / 29 / 33;
-// a request of 1024 trajectories of 19 000 steps 3.7 -> 2.2 ms.
+// a request of 1024 trajectories of 19 000 steps 3.7 -> 2.0 ms.
 constexpr int kTailGroupsMax = 5;       // a quarter of the warps: one scheduler's
 constexpr int kTailMakers = 3;          // noise warps per group
 constexpr int kTailChunk = 3;           // blocks per chunk, one for each of them
@@ -1250,6 +1248,9 @@ __device__ __noinline__ void tail_run(const EngineDev &E, int *held, int groups,
     if (lane == 0) E.warp_kind[gtid >> 5] = warp < groups ? sh.kind[warp] : -1;
 }
 
+// One trajectory per thread runs best as one CTA of 640 threads per SM: 20 warps, five per
+// scheduler, at 96 registers (measured against 512, 576, 672 and 768); two per thread as CTAs
+// of up to 256.
 // kTail: with the packed last trajectories.  Their named barriers count as all 16 of a CTA, which an SM
 // has for four CTAs: small CTAs, which run no groups, get the kernel without (one to four warps: 16, 10,
 // 6 and 5 CTAs per SM; the sweep at 32 / 64 / 128 threads with four: 493 / 821 / 1012 Gstep/s, so:
@@ -1535,7 +1536,7 @@ __device__ __forceinline__ void add_limbs(unsigned long long &lo, unsigned long 
 // nothing with other calls; it runs until its range is done and adds its exact sums and counts to
 // the caller's.  Ranges of equal size differ in length by a few percent, less than the last
 // trajectories take.  Against one event test per step, a full Philox per call and one queue for all
-// CTAs (256 threads each): 200 003 trajectories of 19 000 steps 16.8 -> 6.5 ms.
+// CTAs (256 threads each): 200 003 trajectories of 19 000 steps 17-18 -> 6.0-6.2 ms.
 template <int M, int H, int R>
 __global__ void __launch_bounds__(kSoloThreads, 1) solo_kernel(const __grid_constant__ SoloArgs a) {
     const int warp = static_cast<int>(threadIdx.x >> 5), lane = threadIdx.x & 31;

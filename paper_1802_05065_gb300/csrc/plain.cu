@@ -44,7 +44,8 @@ __device__ __forceinline__ uint32_t hi32(uint64_t x) { return static_cast<uint32
 // sake of one slow lane and a CTA's last trajectories have a scheduler to themselves.
 // Measured, against one trajectory per thread in 128-thread CTAs with noise and update in one
 // chain: 4096 underdamped trajectories of <= 20 000 steps 56.4 -> 21.1 ms (2.8 -> 1.05 us per
-// step; 17.5 ms with F64Pair), 65 536 overdamped ones of 19 000 steps on average 763 -> 226 ms (1.6 -> 5.5 Gstep/s).
+// step; 17.5 ms with F64Pair), 65 536 overdamped ones of 19 000 steps on average 755 -> 239 ms (1.6 -> 5.2 Gstep/s; the
+// longest of them decides: 228-262 ms over six sets).
 constexpr int kF64Warps = 8;
 constexpr int kF64Blocks = 16;                  // Philox blocks per round (fewer for a smaller step budget)
 constexpr int kF64Steps = 4 * kF64Blocks;       // steps per round

@@ -1,7 +1,7 @@
 """Error of the single-precision engine against the double-precision kernel, per workload.
 
-The FP32 engine and the FP64 kernel (the arithmetic of Alg. 1 / Alg. 3 in double precision) integrate the same trajectory ids of the same seed.  The FP32
-uniform is the FP64 one rounded to 23 bits, so both paths see nearly the same noise and the
+The FP32 engine and the FP64 kernel (the arithmetic of Alg. 1 / Alg. 3 in double precision)
+integrate the same trajectory ids of the same seed.  The FP32 uniform is the FP64 one rounded to 23 bits, so both paths see nearly the same noise and the
 per-trajectory difference of the result (escape time or switching bias) isolates the error of
 single precision.  Reported per case: both means and standard errors, the mean paired difference
 and its standard error, the difference of means in combined standard errors, and the
